@@ -10,6 +10,31 @@ struct lbm_s;  // the handle behind lbm_t (lbm_handle.h)
 
 namespace lbm {
 
+// Kernels of one chain of launches overlap their launch with the end of the
+// kernel before: the next grid is set up while the last blocks finish, and
+// every kernel launched this way calls pdl_wait, which returns when the grid
+// before has completed and its writes are visible, before it touches global
+// memory.  No kernel asks for the next one earlier (launch_dependents): blocks
+// placed while the current grid still holds most slots end up unevenly spread
+// over the SMs (FP32 257^2: 2.35 us per step so, 1.92 without; 2.16 without any
+// overlap).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... P, typename... A>
+cudaError_t launch_chain(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, const A&... args) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, P(args)...);
+}
+
 // 0: no force, 1: uniform force only, 2: per-node field (plus the uniform force).
 int force_mode(const lbm_s* h);
 

@@ -21,6 +21,7 @@ template <int MODEL, int STORE, bool ODD, int FORCE, bool WALLS, bool SR = false
 __global__ void __launch_bounds__(kStepBX * kStepBY) step_kernel(const Args a) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    pdl_wait();
     if (x >= a.nx || y >= a.ny) return;
     step_node_split<MODEL, STORE, ODD, FORCE, WALLS, SR>(a, x, y, SR ? round_base(a) : 0u);
 }
@@ -31,6 +32,7 @@ template <int MODEL, int STORE, bool ODD, int FORCE, bool SR>
 __global__ void __launch_bounds__(kStepBX * kStepBY) step_kernel_oop(const Args a) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    pdl_wait();
     if (x >= a.nx || y >= a.ny) return;
     step_node<MODEL, STORE, ODD, FORCE, false, SR, true>(a, x, y, SR ? round_base(a) : 0u);
 }
@@ -41,6 +43,7 @@ template <int MODEL, int STORE, bool ODD, int FORCE, bool WALLS>
 __global__ void __launch_bounds__(kStepBX * kStepBY, 4) step_kernel_pair(const Args a) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = 2 * (blockIdx.y * blockDim.y + threadIdx.y);
+    pdl_wait();
     if (x >= a.nx || y >= a.ny) return;
     const bool two = y + 1 < a.ny;
     if (WALLS && ((x == 0) | (x == a.nx - 1) | (y == 0) | (y + 1 >= a.ny - 1))) {
@@ -71,6 +74,7 @@ __global__ void __launch_bounds__(kVecThreads, ODD ? 8 : 6) step_kernel_vec(cons
     const bool vec = inside && (ODD ? (x0 >= N && x0 + N < a.nx && (!WALLS || (y > 0 && y < a.ny - 1)))
                                     : (x0 + N <= a.nx));
     const unsigned vmask = ODD ? __ballot_sync(0xffffffffu, vec) : 0u;
+    pdl_wait();
     if (vec) {
         step_vec<N, MODEL, STORE, ODD, FORCE, SR>(a, x0, y, vmask, threadIdx.x & 31);
     } else if (inside) {
@@ -94,8 +98,7 @@ static cudaError_t launch_vec(const Args& a, cudaStream_t s) {
     const int vecs = (a.nx + N - 1) / N;
     const dim3 block = fit_block(a.block_x > 0 ? a.block_x : kStepBX, vecs, kVecThreads);
     const dim3 grid((vecs + block.x - 1) / block.x, (a.ny + block.y - 1) / block.y);
-    step_kernel_vec<N, MODEL, STORE, ODD, FORCE, WALLS, SR><<<grid, block, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_chain(step_kernel_vec<N, MODEL, STORE, ODD, FORCE, WALLS, SR>, grid, block, 0, s, a);
 }
 
 template <int MODEL, int STORE, bool ODD, int FORCE, bool WALLS>
@@ -104,9 +107,8 @@ static cudaError_t launch_one(const Args& a, cudaStream_t s) {
         if constexpr ((STORE == LBM_F32 || STORE == LBM_F64) && !WALLS) {
             const dim3 block = fit_block(a.block_x > 0 ? a.block_x : kStepBX, a.nx);
             const dim3 grid((a.nx + block.x - 1) / block.x, (a.ny + block.y - 1) / block.y);
-            if (a.rseed) step_kernel_oop<MODEL, STORE, ODD, FORCE, true><<<grid, block, 0, s>>>(a);
-            else step_kernel_oop<MODEL, STORE, ODD, FORCE, false><<<grid, block, 0, s>>>(a);
-            return cudaGetLastError();
+            if (a.rseed) return launch_chain(step_kernel_oop<MODEL, STORE, ODD, FORCE, true>, grid, block, 0, s, a);
+            return launch_chain(step_kernel_oop<MODEL, STORE, ODD, FORCE, false>, grid, block, 0, s, a);
         }
         return cudaErrorNotSupported;
     }
@@ -114,8 +116,7 @@ static cudaError_t launch_one(const Args& a, cudaStream_t s) {
         if (a.rseed) {  // stochastic rounding of FP32 stores: variant 0 only
             const dim3 block = fit_block(a.block_x > 0 ? a.block_x : kStepBX, a.nx);
             const dim3 grid((a.nx + block.x - 1) / block.x, (a.ny + block.y - 1) / block.y);
-            step_kernel<MODEL, STORE, ODD, FORCE, WALLS, true><<<grid, block, 0, s>>>(a);
-            return cudaGetLastError();
+            return launch_chain(step_kernel<MODEL, STORE, ODD, FORCE, WALLS, true>, grid, block, 0, s, a);
         }
     }
     if constexpr (STORE == LBM_F16DEV || STORE == LBM_BF16DEV) {
@@ -125,8 +126,7 @@ static cudaError_t launch_one(const Args& a, cudaStream_t s) {
             }
             const dim3 block = fit_block(a.block_x > 0 ? a.block_x : kStepBX, a.nx);
             const dim3 grid((a.nx + block.x - 1) / block.x, (a.ny + block.y - 1) / block.y);
-            step_kernel<MODEL, STORE, ODD, FORCE, WALLS, true><<<grid, block, 0, s>>>(a);
-            return cudaGetLastError();
+            return launch_chain(step_kernel<MODEL, STORE, ODD, FORCE, WALLS, true>, grid, block, 0, s, a);
         }
         if constexpr (FORCE != 2) {
             if (a.variant == 2) return launch_vec<4, MODEL, STORE, ODD, FORCE, WALLS, false>(a, s);
@@ -138,13 +138,11 @@ static cudaError_t launch_one(const Args& a, cudaStream_t s) {
         if (a.variant == 1) {
             const int rows = (a.ny + 1) / 2;
             const dim3 grid((a.nx + bx - 1) / bx, (rows + by - 1) / by);
-            step_kernel_pair<MODEL, STORE, ODD, FORCE, WALLS><<<grid, block, 0, s>>>(a);
-            return cudaGetLastError();
+            return launch_chain(step_kernel_pair<MODEL, STORE, ODD, FORCE, WALLS>, grid, block, 0, s, a);
         }
     }
     const dim3 grid((a.nx + bx - 1) / bx, (a.ny + by - 1) / by);
-    step_kernel<MODEL, STORE, ODD, FORCE, WALLS><<<grid, block, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_chain(step_kernel<MODEL, STORE, ODD, FORCE, WALLS>, grid, block, 0, s, a);
 }
 
 template <int MODEL, int STORE, bool ODD, int FORCE>
