@@ -280,14 +280,18 @@ __device__ __forceinline__ void load_node(const Args& a, int x, int y, typename 
         const int r0 = y * a.pitch;
 #pragma unroll
         for (int q = 0; q < 9; ++q) {
-            int w = -1;
-            if (WALLS) w = incoming_wall(a, q, x, y);
-            if (w >= 0) {
-                d[q] = add_wall_term<R>(a, S::dec(plane_ptr(a, f, q)[n]), q, w);
-            } else {
-                const int sx = cx(q) == 1 ? xm : (cx(q) == -1 ? xp : x);
-                const int sr = cy(q) == 1 ? rm : (cy(q) == -1 ? rp : r0);
-                d[q] = S::dec(plane_ptr(a, f, opp(q))[sr + sx]);
+            const int w = WALLS ? incoming_wall(a, q, x, y) : -1;
+            const int sx = cx(q) == 1 ? xm : (cx(q) == -1 ? xp : x);
+            const int sr = cy(q) == 1 ? rm : (cy(q) == -1 ? rp : r0);
+            // a reflected link reads the node's own slot q; one load either way
+            const T* src = w >= 0 ? plane_ptr(a, f, q) + n : plane_ptr(a, f, opp(q)) + (sr + sx);
+            d[q] = S::dec(*src);
+        }
+        if (WALLS) {
+#pragma unroll
+            for (int q = 1; q < 9; ++q) {
+                const int w = incoming_wall(a, q, x, y);
+                if (w >= 0) d[q] = add_wall_term<R>(a, d[q], q, w);
             }
         }
     }
@@ -716,11 +720,12 @@ __device__ __forceinline__ void step_node(const Args& a, int x, int y, unsigned 
 }
 
 // As step_node; with walls, only nodes on the lattice edge take the wall-aware
-// path (an interior node has no wall link and no wrapped neighbour).  rb as in
+// path (an interior node has no wall link and no wrapped neighbour), and only
+// on odd steps: an even step reads and writes the node's own slots.  rb as in
 // store_node (ignored unless SR).
 template <int MODEL, int STORE, bool ODD, int FORCE, bool WALLS, bool SR = false>
 __device__ __forceinline__ void step_node_split(const Args& a, int x, int y, unsigned rb = 0u) {
-    if (WALLS && ((x == 0) | (x == a.nx - 1) | (y == 0) | (y == a.ny - 1)))
+    if (WALLS && ODD && ((x == 0) | (x == a.nx - 1) | (y == 0) | (y == a.ny - 1)))
         step_node<MODEL, STORE, ODD, FORCE, true, SR>(a, x, y, rb);
     else
         step_node<MODEL, STORE, ODD, FORCE, false, SR>(a, x, y, rb);

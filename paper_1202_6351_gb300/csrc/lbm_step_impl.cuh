@@ -17,13 +17,23 @@
 
 namespace lbm {
 
+//
+// With walls, a warp that holds a node on the lattice edge takes the wall-aware
+// path with all its lanes on odd steps: the lanes that need it and the others
+// together cost one update, where a branch per node cost one of each, the whole
+// latency of a launch on a small lattice (FP32 cavity on 101^2).
 template <int MODEL, int STORE, bool ODD, int FORCE, bool WALLS, bool SR = false>
 __global__ void __launch_bounds__(kStepBX * kStepBY) step_kernel(const Args a) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    const bool inside = x < a.nx && y < a.ny;
+    const bool edge = WALLS && ODD &&
+                      __any_sync(0xffffffffu, inside && ((x == 0) | (x == a.nx - 1) | (y == 0) | (y == a.ny - 1)));
     pdl_wait();
-    if (x >= a.nx || y >= a.ny) return;
-    step_node_split<MODEL, STORE, ODD, FORCE, WALLS, SR>(a, x, y, SR ? round_base(a) : 0u);
+    if (!inside) return;
+    const unsigned rb = SR ? round_base(a) : 0u;
+    if (edge) step_node<MODEL, STORE, ODD, FORCE, WALLS && ODD, SR>(a, x, y, rb);
+    else step_node<MODEL, STORE, ODD, FORCE, false, SR>(a, x, y, rb);
 }
 
 // One node per thread from a.f into a.fo (out of place; periodic lattices,
