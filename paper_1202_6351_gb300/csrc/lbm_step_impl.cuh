@@ -22,10 +22,22 @@ namespace lbm {
 // path with all its lanes on odd steps: the lanes that need it and the others
 // together cost one update, where a branch per node cost one of each, the whole
 // latency of a launch on a small lattice (FP32 cavity on 101^2).
-template <int MODEL, int STORE, bool ODD, int FORCE, bool WALLS, bool SR = false>
+//
+// LIN: nodes numbered row by row over the lanes instead of a row per warp, so
+// a narrow or ragged lattice leaves no lanes idle.  FP64 updates are bound by
+// the FP64 pipe, which takes 16 cycles per warp instruction and SM however many
+// lanes are active: full warps, one per CTA so that they spread over all SMs.
+template <int MODEL, int STORE, bool ODD, int FORCE, bool WALLS, bool SR = false, bool LIN = false>
 __global__ void __launch_bounds__(kStepBX * kStepBY) step_kernel(const Args a) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
+    int x, y;
+    if (LIN) {
+        const unsigned n = blockIdx.x * blockDim.x + threadIdx.x;
+        y = int(n / unsigned(a.nx));
+        x = int(n - unsigned(y) * unsigned(a.nx));
+    } else {
+        x = blockIdx.x * blockDim.x + threadIdx.x;
+        y = blockIdx.y * blockDim.y + threadIdx.y;
+    }
     const bool inside = x < a.nx && y < a.ny;
     const bool edge = WALLS && ODD &&
                       __any_sync(0xffffffffu, inside && ((x == 0) | (x == a.nx - 1) | (y == 0) | (y == a.ny - 1)));
@@ -141,6 +153,11 @@ static cudaError_t launch_one(const Args& a, cudaStream_t s) {
         if constexpr (FORCE != 2) {
             if (a.variant == 2) return launch_vec<4, MODEL, STORE, ODD, FORCE, WALLS, false>(a, s);
         }
+    }
+    if constexpr (STORE == LBM_F64) {  // one full warp per CTA
+        const unsigned nodes = unsigned(a.nx) * unsigned(a.ny);
+        return launch_chain(step_kernel<MODEL, STORE, ODD, FORCE, WALLS, false, true>, dim3((nodes + 31) / 32), dim3(32),
+                            0, s, a);
     }
     const dim3 block = fit_block(a.block_x > 0 ? a.block_x : kStepBX, a.nx);
     const int bx = block.x, by = block.y;
