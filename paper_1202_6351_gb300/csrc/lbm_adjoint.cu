@@ -23,7 +23,7 @@
 namespace lbm {
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 128;
 
 template <typename R>
 __device__ __forceinline__ void force_rt(const Args& a, int force, int x, int y, R& Fx, R& Fy) {
@@ -94,23 +94,43 @@ __global__ void __launch_bounds__(kThreads) adj_final_kernel(const Args a, bool 
 // on the first reverse step of a checkpoint segment (`first`), added after
 // that; adj_fold_kernel adds each segment's sum into the FP64 gradient (for
 // FP64 storage gs is the FP64 gradient itself and `first` is false).
-// Each thread takes kAdjRows node rows (y0, y0 + 1, ...) of its column and
-// sums their rate adjoints in registers, so the block reduction of the six
-// sums runs once per kAdjRows nodes.
+// A block takes kAdjRows rows of nodes, RPT rows per thread (one after the
+// other).  The kernel is bound by the latency of its 18 loads and of the
+// transposed collision.  On a small lattice the nodes have to be in flight
+// together: RPT = 1 (four rows per thread left 80 % of the warp slots of 512^2
+// empty).  From 2^20 nodes on, where every slot is filled anyway, RPT = 4 spares
+// three of four block reductions (2048^2: 273 us per differentiated step, forward
+// and recompute included, against 285 with RPT = 1).  Blocks of 128 threads, seven
+// per SM (72 registers): 1024^2 67.8 us, 70.8 with eight, 76 with six.
+// us per differentiated step, before -> now: 128^2 16.4 -> 6.3, 512^2 27.7 -> 21.2,
+// 1024^2 78.7 -> 67.8, 2048^2 280 -> 270.
+// The six rate sums add the four rows of a column in row order (in registers or
+// through shared memory), then the 32 columns of a warp by shuffles, in the
+// arithmetic type, and then in FP64 over time in a slot of the warp's own; the
+// six go to six lanes first, since an FP64 instruction costs 64 cycles whether
+// one lane works or all.  adj_rates_kernel adds the slots up once at the end.
+// Atomic additions onto six words are serialised at the L2 (two per 256 nodes:
+// 82 ms for the 100 steps of a 2048^2 run that take 59).
 constexpr int kAdjRows = 4;
+constexpr int adj_cols(int rpt) { return kThreads * rpt / kAdjRows; }
+inline bool adj_serial_rows(const Args& a) { return (long long)a.nx * a.ny >= (1LL << 20); }
 
-template <int ST>
-__global__ void __launch_bounds__(kThreads, ST == LBM_F32 ? 4 : 1) adj_step_kernel(const Args a, bool odd, int force,
+template <int ST, int RPT>
+__global__ void __launch_bounds__(kThreads, ST == LBM_F32 ? 7 : 1) adj_step_kernel(const Args a, bool odd, int force,
                                                             const typename Store<ST>::R* __restrict__ lin,
                                                             typename Store<ST>::R* __restrict__ lout,
                                                             typename Store<ST>::R* __restrict__ gs, bool first,
                                                             double* gc) {
     using R = typename Store<ST>::R;
-    const int x = blockIdx.x * kThreads + threadIdx.x, y0 = blockIdx.y * kAdjRows;
+    constexpr int COLS = adj_cols(RPT);
+    __shared__ R rows[RPT == 1 ? 6 : 1][RPT == 1 ? kThreads : 1];
+    const int tid = threadIdx.x, col = tid % COLS, lane = tid & 31;
+    const int x = blockIdx.x * COLS + col, y0 = blockIdx.y * kAdjRows + tid / COLS;
     R c[6] = {0, 0, 0, 0, 0, 0};
+    pdl_wait();
     if (x < a.nx) {
         const int xm = x > 0 ? x - 1 : a.nx - 1, xp = x < a.nx - 1 ? x + 1 : 0;
-        const int yend = min(y0 + kAdjRows, a.ny);
+        const int yend = min(y0 + RPT, a.ny);
 #pragma unroll 1
         for (int y = y0; y < yend; ++y) {
             const Coef<R> co(a);
@@ -143,7 +163,41 @@ __global__ void __launch_bounds__(kThreads, ST == LBM_F32 ? 4 : 1) adj_step_kern
             for (int k = 0; k < 6; ++k) c[k] += g.c[k];
         }
     }
-    block_atomic_add<6>(c, gc);
+    if constexpr (RPT == 1) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) rows[k][tid] = c[k];
+        __syncthreads();
+        if (tid >= COLS) return;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+#pragma unroll
+            for (int r = 1; r < kAdjRows; ++r) c[k] += rows[k][r * COLS + col];
+        }
+    }
+    R mine = 0;  // lane k: the warp's sum k
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        for (int o = 16; o > 0; o >>= 1) c[k] += __shfl_down_sync(0xffffffffu, c[k], o);
+        const R t = __shfl_sync(0xffffffffu, c[k], 0);
+        if (lane == k) mine = t;
+    }
+    if (lane < 6)
+        gc[6 * ((COLS / 32) * (size_t(blockIdx.y) * gridDim.x + blockIdx.x) + (tid >> 5)) + lane] += double(mine);
+}
+
+// acc[k] = the sum of the n slots' k-th rate sums, one block per k, in a fixed order.
+__global__ void __launch_bounds__(kThreads) adj_rates_kernel(const double* __restrict__ gc, size_t n, double* acc) {
+    __shared__ double sh[kThreads / 32];
+    double v = 0.0;
+    for (size_t i = threadIdx.x; i < n; i += kThreads) v += gc[6 * i + blockIdx.x];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < kThreads / 32; ++w) t += sh[w];
+        acc[blockIdx.x] = t;
+    }
 }
 
 __device__ __forceinline__ double phi(int e, double u) {
@@ -207,9 +261,15 @@ Args at_step(const Args& a, long t) {
     return ak;
 }
 
+// Slots of the rate sums of a lattice's reverse steps (one per warp of columns and block of rows).
+size_t adj_slots(const Args& a) {
+    const int cols = adj_cols(adj_serial_rows(a) ? kAdjRows : 1);
+    return size_t(cols / 32) * ((a.nx + cols - 1) / cols) * ((a.ny + kAdjRows - 1) / kAdjRows);
+}
+
 template <int ST>
 cudaError_t run_reverse(lbm_s* h, long nsteps, long every, const double* rho, const double* u0, const double* target,
-                        char* ckpt, char* seg, void* lam0, void* lam1, double* gF, float* gseg, double* acc,
+                        char* ckpt, char* seg, void* lam0, void* lam1, double* gF, float* gseg, double* acc, double* gc,
                         double* gu0) {
     using R = typename Store<ST>::R;
     const Args& a = h->a;
@@ -258,13 +318,16 @@ cudaError_t run_reverse(lbm_s* h, long nsteps, long every, const double* rho, co
             if ((e = launch_step_any(ak, h->store, h->model, (n0 + k - 1) & 1, fm, false, s)) != cudaSuccess) return e;
         }
         R* gs = ST == LBM_F64 ? reinterpret_cast<R*>(gF) : reinterpret_cast<R*>(gseg);
-        const dim3 agrid(grid.x, (a.ny + kAdjRows - 1) / kAdjRows);
+        const bool serial = adj_serial_rows(a);
+        const int cols = adj_cols(serial ? kAdjRows : 1);
+        const dim3 agrid((a.nx + cols - 1) / cols, (a.ny + kAdjRows - 1) / kAdjRows);
         for (long k = len - 1; k >= 0; --k) {
             Args ak = a;
             ak.f = state(k);
             const bool first = ST != LBM_F64 && k == len - 1;
-            adj_step_kernel<ST><<<agrid, kThreads, 0, s>>>(ak, (n0 + k) & 1, fm, cur, nxt, gs, first, acc + 1);
-            if ((e = cudaGetLastError()) != cudaSuccess) return e;
+            if ((e = launch_chain(serial ? adj_step_kernel<ST, kAdjRows> : adj_step_kernel<ST, 1>, agrid, dim3(kThreads), 0, s, ak, bool((n0 + k) & 1), fm, cur, nxt,
+                                  gs, first, gc)) != cudaSuccess)
+                return e;
             std::swap(cur, nxt);
         }
         if (ST != LBM_F64) {
@@ -273,6 +336,8 @@ cudaError_t run_reverse(lbm_s* h, long nsteps, long every, const double* rho, co
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
     }
+    adj_rates_kernel<<<6, kThreads, 0, s>>>(gc, adj_slots(a), acc + 1);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
     adj_init_kernel<ST><<<grid, kThreads, 0, s>>>(a, fm, rho, u0, cur, gu0, gF);
     return cudaGetLastError();
 }
@@ -316,9 +381,11 @@ extern "C" int lbm_adjoint_run(lbm_t h, long nsteps, long every, const double* r
     void* lam0 = alloc(lam_bytes);
     void* lam1 = alloc(lam_bytes);
     double* acc = static_cast<double*>(alloc(7 * sizeof(double)));
+    const size_t gc_bytes = 6 * adj_slots(h->a) * sizeof(double);
+    double* gc = static_cast<double*>(alloc(gc_bytes));
     double* gF = grad_force ? grad_force : static_cast<double*>(alloc(2 * n * sizeof(double)));
     float* gseg = h->store == LBM_F64 ? nullptr : static_cast<float*>(alloc(2 * n * sizeof(float)));
-    if (!ckpt || !seg || !lam0 || !lam1 || !acc || !gF || (h->store != LBM_F64 && !gseg)) {
+    if (!ckpt || !seg || !lam0 || !lam1 || !acc || !gc || !gF || (h->store != LBM_F64 && !gseg)) {
         release();
         cudaGetLastError();
         if (prev >= 0 && prev != h->device) cudaSetDevice(prev);
@@ -326,12 +393,13 @@ extern "C" int lbm_adjoint_run(lbm_t h, long nsteps, long every, const double* r
                          ((nck + std::max(1L, seglen - 1)) * SB + 2 * lam_bytes) / 1e6);
     }
     cudaError_t e = cudaMemsetAsync(acc, 0, 7 * sizeof(double), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(gc, 0, gc_bytes, s);
     if (e == cudaSuccess) {
         e = h->store == LBM_F64
                 ? run_reverse<LBM_F64>(h, nsteps, every, rho, u0, u_target, ckpt, seg, lam0, lam1, gF, gseg, acc,
-                                       grad_u0)
+                                       gc, grad_u0)
                 : run_reverse<LBM_F32>(h, nsteps, every, rho, u0, u_target, ckpt, seg, lam0, lam1, gF, gseg, acc,
-                                       grad_u0);
+                                       gc, grad_u0);
     }
     double host[7] = {0, 0, 0, 0, 0, 0, 0};
     if (e == cudaSuccess) e = cudaMemcpyAsync(host, acc, sizeof host, cudaMemcpyDeviceToHost, s);
