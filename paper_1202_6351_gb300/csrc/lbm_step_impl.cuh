@@ -81,15 +81,22 @@ __global__ void __launch_bounds__(kStepBX * kStepBY, 4) step_kernel_pair(const A
 // The CTA is bx x by threads with bx a multiple of 32, so the lanes of a warp
 // hold consecutive vectors of one row (step_vec exchanges elements between
 // neighbouring lanes on odd steps).
-// Register budget per parity, as measured: the even step keeps all nine planes
-// aligned and spills at 64 registers, so it gets 80 (6 CTAs of 128 threads per
-// SM); the odd step runs faster with more warps at 64 (8 CTAs per SM).  CTAs of
-// 128 threads rather than 256 run the four-node kernel 3-4 % faster (FP16 on
-// 4096^2: 145.5 against 140.6 GLUPS).
+// Register budget per parity, as measured, in CTAs of 128 threads per SM
+// (CTAs of 256 run 3-4 % slower).  Node pairs (the unforced cascaded collision):
+// five on the even step, where six (80 registers) spill (98.5 against 102 us per
+// FP16 4096^2 launch); on the odd step seven, six with stochastic rounding, which
+// keeps two random words per pair (4096^2: 109.8 us per step with seven, 108.5
+// with six, 115 with eight; cavity 8192^2 419, 431, 419).  Single nodes: the even
+// step spills at 64 registers and gets 80 (six); the odd step runs faster with
+// more warps at 64 (eight).
 constexpr int kVecThreads = 128;
+constexpr bool vec_pairs(int model, int force) { return model == LBM_CASCADED && force == 0; }
+constexpr int vec_blocks(bool pairs, bool odd, bool sr) {
+    return pairs ? (odd ? (sr ? 6 : 7) : 5) : (odd ? 8 : 6);
+}
 
 template <int N, int MODEL, int STORE, bool ODD, int FORCE, bool WALLS, bool SR>
-__global__ void __launch_bounds__(kVecThreads, ODD ? 8 : 6) step_kernel_vec(const Args a) {
+__global__ void __launch_bounds__(kVecThreads, vec_blocks(vec_pairs(MODEL, FORCE), ODD, SR)) step_kernel_vec(const Args a) {
     const int x0 = N * (blockIdx.x * blockDim.x + threadIdx.x);
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const bool inside = x0 < a.nx && y < a.ny;
@@ -98,7 +105,8 @@ __global__ void __launch_bounds__(kVecThreads, ODD ? 8 : 6) step_kernel_vec(cons
     const unsigned vmask = ODD ? __ballot_sync(0xffffffffu, vec) : 0u;
     pdl_wait();
     if (vec) {
-        step_vec<N, MODEL, STORE, ODD, FORCE, SR>(a, x0, y, vmask, threadIdx.x & 31);
+        if constexpr (vec_pairs(MODEL, FORCE)) step_vec_pair<STORE, ODD, SR>(a, x0, y, vmask, threadIdx.x & 31);
+        else step_vec<N, MODEL, STORE, ODD, FORCE, SR>(a, x0, y, vmask, threadIdx.x & 31);
     } else if (inside) {
         const int x1 = min(x0 + N, a.nx);
         const unsigned rb = SR ? round_base(a) : 0u;

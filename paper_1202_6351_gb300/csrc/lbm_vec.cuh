@@ -38,6 +38,7 @@
 #include <stdint.h>
 
 #include "lbm_device.cuh"
+#include "lbm_pair.cuh"
 
 namespace lbm {
 
@@ -232,6 +233,113 @@ __device__ __forceinline__ void step_vec(const Args& a, int x0, int y, unsigned 
                 base[N - 2] = os1[p];
             }
             if (!left_ok) base[-1] = os0[p];
+        }
+    }
+}
+
+// Stochastic rounding of two values into one word (element 0 in the low half),
+// as two StochasticRound<STORE>::enc; r0 and r1 are the nodes' random words.
+template <int STORE>
+__device__ __forceinline__ uint32_t enc_sr2(float2 v, unsigned r0, unsigned r1) {
+    if constexpr (STORE == LBM_F16DEV) {
+        const float lo = __uint_as_float(__float_as_uint(v.x) + (r0 >> 19)), hi = __uint_as_float(__float_as_uint(v.y) + (r1 >> 19));
+        uint32_t w;
+        asm("cvt.rz.f16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(hi), "f"(lo));
+        return w;
+    } else {
+        return __byte_perm(__float_as_uint(v.x) + (r0 >> 16), __float_as_uint(v.y) + (r1 >> 16), 0x7632);
+    }
+}
+
+// step_vec for the cascaded collision without a force: two node pairs in packed
+// FP32x2 arithmetic (collide_cascaded_pair, value for value the scalar
+// collision).  The populations stay packed two to a word from load to store: a
+// pair of an unshifted plane is one word of the aligned vector, a pair of a
+// shifted plane the upper half of one word and the lower half of the next (one
+// byte permute), and the results replace the words they came from.
+//
+// Thread instructions per node 148 -> 104 (even step, 96 registers, 70 % of HBM
+// peak, bound by load latency) and 204 -> 184 (odd step: the narrow accesses of
+// the first and last lane of a warp, which every warp issues).  us per step,
+// before -> now: FP16 periodic 4096^2 114.6 -> 109.8, cavity 8192^2 464 -> 419,
+// cavity 1025^2 10.8 -> 9.5, BF16 4096^2 118.7 -> 108.0, FP16 stochastic 2048^2
+// 31.0 -> 30.5.  Gathering the narrow accesses of a side under one branch issued
+// as much and ran 2 % slower.
+template <int STORE, bool ODD, bool SR>
+__device__ __forceinline__ void step_vec_pair(const Args& a, int x0, int y, unsigned vmask, int lane) {
+    using H = Half16<STORE>;
+    unsigned short* __restrict__ f = static_cast<unsigned short*>(a.f);
+    const int r0 = y * a.pitch;
+    const int rm = (y > 0 ? y - 1 : a.ny - 1) * a.pitch, rp = (y < a.ny - 1 ? y + 1 : 0) * a.pitch;
+    const bool left_ok = ODD && lane > 0 && ((vmask >> (lane - 1)) & 1u);
+    const bool right_ok = ODD && lane < 31 && ((vmask >> (lane + 1)) & 1u);
+    const int o0 = r0 + x0, om = rm + x0, op = rp + x0;
+    auto vec = [&](int p) { return plane_ptr(a, f, p) + (ODD ? (cy(p) == 1 ? op : (cy(p) == -1 ? om : o0)) : o0); };
+
+    uint32_t w[9][2];  // word k of plane p: the pair (x0 + s + 2 k, x0 + s + 2 k + 1), s = e_p,x on odd steps, else 0
+#pragma unroll
+    for (int p = 0; p < 9; ++p) VecN<4>::load(vec(p), w[p]);
+    if (ODD) {
+#pragma unroll
+        for (int p = 0; p < 9; ++p) {
+            const uint32_t w0 = w[p][0], w1 = w[p][1];
+            if (cx(p) == 1) {  // element 4 is the right neighbour's first
+                uint32_t r = __shfl_down_sync(vmask, w0, 1);
+                if (!right_ok) r = vec(p)[4];
+                w[p][0] = __byte_perm(w0, w1, 0x5432);
+                w[p][1] = __byte_perm(w1, r, 0x5432);
+            } else if (cx(p) == -1) {  // element -1 is the left neighbour's last
+                uint32_t r = __shfl_up_sync(vmask, w1, 1);
+                if (!left_ok) r = static_cast<uint32_t>(vec(p)[-1]) << 16;
+                w[p][0] = __byte_perm(r, w0, 0x5432);
+                w[p][1] = __byte_perm(w0, w1, 0x5432);
+            }
+        }
+    }
+    const unsigned rbase = SR ? round_base(a) : 0u;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        float2 d[9];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            const uint32_t v = w[ODD ? opp(q) : q][k];
+            d[q] = make_float2(H::lo(v), H::hi(v));
+        }
+        collide_cascaded_pair(d, a.kf);
+        const unsigned n0 = SR ? round_node(a, rbase, x0 + 2 * k, y) : 0u, n1 = SR ? round_node(a, rbase, x0 + 2 * k + 1, y) : 0u;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            const unsigned o = static_cast<unsigned>(q) * kRoundStride;
+            w[ODD ? q : opp(q)][k] = SR ? enc_sr2<STORE>(d[q], n0 + o, n1 + o) : H::pack(d[q].x, d[q].y);
+        }
+    }
+#pragma unroll
+    for (int p = 0; p < 9; ++p) {
+        unsigned short* base = vec(p);
+        const uint32_t w0 = w[p][0], w1 = w[p][1];
+        const int s = ODD ? cx(p) : 0;
+        if (s == 0) {
+            VecN<4>::store(base, w[p]);
+        } else if (s == 1) {  // pairs (1, 2), (3, 4): the aligned vector takes the left neighbour's element 4 first
+            const uint32_t r = __shfl_up_sync(vmask, w1, 1);
+            const uint32_t v[2] = {__byte_perm(r, w0, 0x5432), __byte_perm(w0, w1, 0x5432)};
+            if (left_ok) {
+                VecN<4>::store(base, v);
+            } else {
+                base[1] = static_cast<unsigned short>(w0);
+                store_words<1>(base + 2, v + 1);
+            }
+            if (!right_ok) base[4] = static_cast<unsigned short>(w1 >> 16);
+        } else {  // pairs (-1, 0), (1, 2): the aligned vector ends with the right neighbour's element -1
+            const uint32_t r = __shfl_down_sync(vmask, w0, 1);
+            const uint32_t v[2] = {__byte_perm(w0, w1, 0x5432), __byte_perm(w1, r, 0x5432)};
+            if (right_ok) {
+                VecN<4>::store(base, v);
+            } else {
+                store_words<1>(base, v);
+                base[2] = static_cast<unsigned short>(w1 >> 16);
+            }
+            if (!left_ok) base[-1] = static_cast<unsigned short>(w0);
         }
     }
 }
