@@ -13,6 +13,7 @@
 #include "lbm.h"
 #include "lbm_fused.cuh"
 #include "lbm_internal.h"
+#include "lbm_multi.cuh"
 #include "lbm_handle.h"
 
 using lbm::Args;
@@ -137,17 +138,17 @@ EncodeTiledFn encode_tiled() {
     return fn;
 }
 
-template <int ST>
-void fused_box(cuuint32_t box[3]) {
-    box[0] = lbm::FusedGeom<ST>::BW;
-    box[1] = lbm::FusedGeom<ST>::BH;
+template <class G>
+void tile_box(cuuint32_t box[3]) {
+    box[0] = G::BW;
+    box[1] = G::BH;
     box[2] = 9;
 }
 
 // TMA descriptor of a population array of the lattice: a 3-D tensor
 // [9][ny][nx] (x fastest, row pitch `pitch`, plane pitch * ny), box = the
-// fused kernel's region; coordinates beyond nx or ny read zeros.
-cudaError_t encode_map(const lbm_s* h, void* base, CUtensorMap* map) {
+// region of the two-step (or multi-step) kernel; coordinates beyond nx or ny read zeros.
+cudaError_t encode_map(const lbm_s* h, void* base, bool multi, CUtensorMap* map) {
     EncodeTiledFn fn = encode_tiled();
     if (!fn) return cudaErrorNotSupported;
     const size_t es = elem_size(h->store);
@@ -156,10 +157,10 @@ cudaError_t encode_map(const lbm_s* h, void* base, CUtensorMap* map) {
     cuuint32_t box[3];
     CUtensorMapDataType type;
     if (h->store == LBM_F32) {
-        fused_box<LBM_F32>(box);
+        multi ? tile_box<lbm::MultiLarge<LBM_F32>>(box) : tile_box<lbm::FusedGeom<LBM_F32>>(box);
         type = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     } else {
-        fused_box<LBM_F16DEV>(box);
+        multi ? tile_box<lbm::MultiLarge<LBM_F16DEV>>(box) : tile_box<lbm::FusedGeom<LBM_F16DEV>>(box);
         type = CU_TENSOR_MAP_DATA_TYPE_UINT16;
     }
     const cuuint32_t estr[3] = {1, 1, 1};
@@ -175,6 +176,11 @@ bool fused_active(const lbm_s* h) {
     return h->a.variant == 3 && h->store != LBM_F64 && h->a.nx >= 4 && h->a.ny >= 4 && h->check_every == 0;
 }
 
+// Variant 3 runs the multi-step kernel (lbm_multi.cuh) where its node pairs apply.
+bool multi_active(const lbm_s* h) {
+    return fused_active(h) && h->model == LBM_CASCADED && force_mode(h) == 0 && !h->a.rseed;
+}
+
 // Second population array, descriptors and error word (first use of variant 3).
 cudaError_t ensure_fused(lbm_s* h) {
     cudaError_t e = cudaSuccess;
@@ -185,8 +191,10 @@ cudaError_t ensure_fused(lbm_s* h) {
     }
     // The two arrays only ever swap roles, so one descriptor each, made once.
     if (e == cudaSuccess && !h->tmap_ptr[0]) {
-        e = encode_map(h, h->state, &h->tmap[0]);
-        if (e == cudaSuccess) e = encode_map(h, h->state_alt, &h->tmap[1]);
+        e = encode_map(h, h->state, false, &h->tmap[0]);
+        if (e == cudaSuccess) e = encode_map(h, h->state_alt, false, &h->tmap[1]);
+        if (e == cudaSuccess) e = encode_map(h, h->state, true, &h->mmap[0]);
+        if (e == cudaSuccess) e = encode_map(h, h->state_alt, true, &h->mmap[1]);
         if (e == cudaSuccess) {
             h->tmap_ptr[0] = h->state;
             h->tmap_ptr[1] = h->state_alt;
@@ -212,16 +220,29 @@ void swap_arrays(lbm_s* h) {
     h->a.f = h->state;
 }
 
-// Two fused steps t, t + 1 (t even) outside a graph.
-cudaError_t launch_pair_at(lbm_s* h, long t) {
+// Fused steps from the even step t, at most `left` (>= 2), outside a graph;
+// *took is the number of steps of the launch.
+cudaError_t launch_fused_at(lbm_s* h, long t, long left, int* took) {
     lbm::Args a = h->a;
-    if (a.rseed) {
-        a.rbase = lbm::round_hash(a.rseed, static_cast<unsigned long long>(t));
-        a.rbase1 = lbm::round_hash(a.rseed, static_cast<unsigned long long>(t + 1));
-        a.rtable = nullptr;
-        a.tstep = 0;
+    cudaError_t e;
+    if (multi_active(h)) {
+        *took = left >= lbm::kMultiSteps ? lbm::kMultiSteps : 2;
+        const CUtensorMap& map = h->mmap[h->tmap_ptr[0] == a.f ? 0 : 1];
+        switch (h->store) {
+            case LBM_F32: e = lbm::launch_multi_f32(map, a, h->state_alt, h->d_err, *took, h->stream); break;
+            case LBM_BF16DEV: e = lbm::launch_multi_bf16(map, a, h->state_alt, h->d_err, *took, h->stream); break;
+            default: e = lbm::launch_multi_f16(map, a, h->state_alt, h->d_err, *took, h->stream); break;
+        }
+    } else {
+        *took = 2;
+        if (a.rseed) {
+            a.rbase = lbm::round_hash(a.rseed, static_cast<unsigned long long>(t));
+            a.rbase1 = lbm::round_hash(a.rseed, static_cast<unsigned long long>(t + 1));
+            a.rtable = nullptr;
+            a.tstep = 0;
+        }
+        e = launch_fused(h, a, h->state_alt, h->stream);
     }
-    cudaError_t e = launch_fused(h, a, h->state_alt, h->stream);
     if (e == cudaSuccess) swap_arrays(h);
     return e;
 }
@@ -239,7 +260,11 @@ int fused_error(lbm_s* h) {
 
 // Steps per graph replay: a multiple of 4 with fused steps (an even number of
 // fused launches ends on the array the graph started from).
-int graph_len(const lbm_s* h) { return fused_active(h) ? (h->graph_steps / 4) * 4 : h->graph_steps; }
+// Launches of the multi-step kernel are long enough to be queued one by one.
+int graph_len(const lbm_s* h) {
+    if (multi_active(h)) return 0;
+    return fused_active(h) ? (h->graph_steps / 4) * 4 : h->graph_steps;
+}
 
 // rtable[k] = the hash of (seed, t0 + k) for the k-th launch of a graph replay.
 __global__ void fill_round_table(unsigned* rtable, unsigned long long seed, unsigned long long t0, int n) {
@@ -575,8 +600,9 @@ int lbm_tune(lbm_t h, int trial_steps, float ms[LBM_NUM_VARIANTS]) {
         cudaError_t e = cudaSuccess;
         for (long t = h->t + k0, end = h->t + k0 + count; t < end && e == cudaSuccess;) {
             if (fused_active(h) && (t & 1) == 0 && end - t >= 2) {
-                e = launch_pair_at(h, t);
-                t += 2;
+                int took = 0;
+                e = launch_fused_at(h, t, end - t, &took);
+                t += took;
             } else {
                 e = launch_step_at(h, (t & 1) != 0, t);
                 t += 1;
@@ -723,9 +749,10 @@ int lbm_step(lbm_t h, long n) {
             continue;
         }
         if (fused && (h->t & 1) == 0 && n - s >= 2) {
-            LBM_CUDA(launch_pair_at(h, h->t), "fused step launch");
-            h->t += 2;
-            s += 2;
+            int took = 0;
+            LBM_CUDA(launch_fused_at(h, h->t, n - s, &took), "fused step launch");
+            h->t += took;
+            s += took;
             continue;
         }
         LBM_CUDA(launch_step(h, (h->t & 1) != 0), "step kernel launch");

@@ -39,7 +39,7 @@ struct lbm_s {
     // the ping-pong, a TMA descriptor of each array (tmap[k] describes
     // tmap_ptr[k]) and the kernels' error word.  Allocated on first use.
     void* state_alt = nullptr;
-    CUtensorMap tmap[2];
+    CUtensorMap tmap[2], mmap[2];  // boxes of the two-step and of the multi-step kernel
     void* tmap_ptr[2] = {nullptr, nullptr};
     int* d_err = nullptr;
 };

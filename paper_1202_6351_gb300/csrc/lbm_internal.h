@@ -60,6 +60,12 @@ cudaError_t launch_fused_bf16(const CUtensorMap& map, const Args& a, void* out, 
 cudaError_t launch_fused_f16(const CUtensorMap& map, const Args& a, void* out, int* err, int model, int force,
                              bool walls, cudaStream_t s);
 
+// 2 or 4 steps of the unforced cascaded collision with round to nearest
+// (lbm_multi.cuh) from a.f (natural layout, even step) into `out`; `map` describes a.f.
+cudaError_t launch_multi_f32(const CUtensorMap& map, const Args& a, void* out, int* err, int steps, cudaStream_t s);
+cudaError_t launch_multi_bf16(const CUtensorMap& map, const Args& a, void* out, int* err, int steps, cudaStream_t s);
+cudaError_t launch_multi_f16(const CUtensorMap& map, const Args& a, void* out, int* err, int steps, cudaStream_t s);
+
 // Auxiliary kernels (lbm_aux.cu); every field argument is dense [..][ny][nx] FP64 device memory.
 cudaError_t launch_init(const Args& a, int store, int model, int force, const double* rho, const double* u,
                         cudaStream_t s);

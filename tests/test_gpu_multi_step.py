@@ -1,0 +1,50 @@
+"""Variant 3 with up to four steps per launch (csrc/lbm_multi.cuh, unforced
+cascaded collision, round to nearest) against one step per launch: the states
+are bit for bit the same.  Sizes sit at the edges of the 32 x 16 and 56 x 40
+tiles and of the size rule between them, and below the four-node halo; step
+counts cover launches of four and two steps and single steps at either end."""
+import numpy as np
+import pytest
+
+from paper_1202_6351_gb300 import lbm, workloads
+
+pytestmark = pytest.mark.gpu
+
+P, BB, MW = lbm.PERIODIC, lbm.BOUNCEBACK, lbm.MOVING_WALL
+EDGES = {
+    "periodic": ((P, P, P, P), (0, 0, 0, 0)),
+    "cavity": ((MW, BB, MW, MW), (0.02, 0, -0.03, 0.1)),
+    "channel_x": ((P, P, BB, MW), (0, 0, 0, 0.05)),
+    "channel_y": ((BB, MW, P, P), (0, 0.04, 0, 0)),
+}
+SHAPES = [(4, 4), (5, 7), (31, 17), (32, 16), (33, 18), (65, 5), (600, 599),            # 32 x 16 tiles
+          (600, 600), (617, 603), (672, 560), (673, 561), (7, 52001), (9002, 41)]       # 56 x 40 tiles
+
+
+@pytest.fixture(scope="module", autouse=True)
+def cuda():
+    import torch
+
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    torch.cuda.set_device(0)
+    yield
+
+
+@pytest.mark.parametrize("store", [lbm.F32, lbm.F16DEV, lbm.BF16DEV], ids=["f32", "f16", "bf16"])
+@pytest.mark.parametrize("edges", list(EDGES))
+@pytest.mark.parametrize("shape", SHAPES, ids=[f"{a}x{b}" for a, b in SHAPES])
+def test_multi_step_launches_are_bitwise_equal_to_single_steps(shape, edges, store):
+    nx, ny = shape
+    kinds, speeds = EDGES[edges]
+    rho, u = workloads.random_fields(nx + 7 * ny, nx, ny, u_amp=0.03, rho_amp=0.01)
+    states = {}
+    for variant in (0, 3):
+        with lbm.Lattice(nx, ny, (1.1, 1.7, 1.7, 1.0, 1.2, 0.9), edges=kinds, wall_u=speeds, store=store) as L:
+            L.set_variant(variant).init(rho, u)
+            states[variant] = []
+            for n in (4, 2, 1, 7, 10):  # launches of 4; 2; 1; 1 + 4 + 2; 4 + 4 + 2 steps
+                L.step(n)
+                states[variant].append(L.get_f())
+            assert L.time == 24
+    for a, b in zip(states[0], states[3]):
+        np.testing.assert_array_equal(a, b)
