@@ -313,13 +313,15 @@ int lbm_batch_set_graph_steps(lbm_batch_t b, int steps);
  * timed out waiting for its tile load (the states are then invalid). */
 int lbm_batch_sync(lbm_batch_t b);
 
-/* Two steps per launch for the whole batch (on != 0): one CTA per 64 x 16
- * tile of any lattice takes both steps of the tile in shared memory (the tile
- * body of lbm_set_variant's variant 3, with its storage kind, edges, force and
- * rounding), so the populations cross HBM once per two steps.  Every lattice
+/* Several steps per launch for the whole batch (on != 0): one CTA per
+ * tile of any lattice takes the steps of the tile in shared memory (the tile
+ * bodies of lbm_set_variant's variant 3, with its storage kind, edges, force and
+ * rounding), so the populations cross HBM once per launch: four steps on 56 x 40
+ * tiles if every lattice of the batch admits that (the cascaded collision, no
+ * force, round to nearest), else two on 64 x 16 tiles.  Every lattice
  * gets a second population array (allocated here, kept by the lattice) and
- * the arrays trade roles at every launch.  lbm_batch_step then takes pairs of
- * steps from even steps and single batched steps for an odd start or end; a
+ * the arrays trade roles at every launch.  lbm_batch_step then takes such
+ * launches from even steps and single batched steps for an odd start or end; a
  * call whose lattices are at steps of different parity takes single steps
  * only.  Each launch runs one kernel per class of lattice (storage kind,
  * walls, force, rounding) on streams of the batch's own, forked from and

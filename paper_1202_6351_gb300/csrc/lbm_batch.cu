@@ -1,7 +1,7 @@
 // lbm_batch.cu -- many independent lattices advanced together: one kernel
 // launch per time step for all of them (a persistent grid walking a tile list,
-// or one CTA per tile), or one launch per two steps for each class of lattice
-// (lbm_batch_fused.cuh), CUDA graphs of `graph_steps` steps, and an autotuner
+// or one CTA per tile), or one launch per two or four steps for each class of
+// lattice (lbm_batch_fused.cuh), CUDA graphs of `graph_steps` steps, and an autotuner
 // that picks the tile shape, the order of the work list and the scheduling
 // policy by timing them on the batch itself.
 #include <algorithm>
@@ -26,6 +26,9 @@ cudaError_t launch_batch_fused_bgk(int, int, const BatchDomain*, const BatchPair
                                    int, int*, cudaStream_t);
 cudaError_t launch_batch_fused_rawmrt(int, int, const BatchDomain*, const BatchPair*, const int*, int, const unsigned*,
                                       int, int, int*, cudaStream_t);
+
+cudaError_t launch_batch_multi_cascaded(int, int, const BatchDomain*, const BatchPair*, const int*, int, int, int*,
+                                        cudaStream_t);
 
 // rtab[d * rstride + k] = the hash of (seed, t + base + k) of domain d, for the
 // k-th launch of a sequence that starts `base` steps after the domains' counts t.
@@ -78,7 +81,10 @@ struct lbm_batch_s {
     // (class_first[c] .. class_first[c + 1] - 1 are the tiles of class c) for
     // the classes in cls2; the kernels of the second and later classes of a
     // launch run on branch streams forked from the batch stream.
-    bool two_step = false;
+    // A batch whose lattices all take the multi-step tile (unforced cascaded,
+    // round to nearest: `multi`) lists 56 x 40 tiles and takes four steps per
+    // launch.
+    bool two_step = false, multi = false;
     lbm::BatchPair* h_pairs = nullptr;
     lbm::BatchPair* d_pairs = nullptr;
     int* d_tiles2 = nullptr;
@@ -185,6 +191,8 @@ cudaError_t refresh_domains(lbm_batch_s* b) {
             P.arr[1] = h->state_alt;
             P.map[0] = lbm_tensor_map(h, h->state);
             P.map[1] = lbm_tensor_map(h, h->state_alt);
+            P.mmap[0] = lbm_multi_map(h, h->state);
+            P.mmap[1] = lbm_multi_map(h, h->state_alt);
         }
         e = cudaMemcpyAsync(b->d_pairs, b->h_pairs, b->doms.size() * sizeof(lbm::BatchPair), cudaMemcpyHostToDevice,
                             b->stream);
@@ -273,11 +281,30 @@ std::vector<int> domain_classes(const lbm_batch_s* b) {
     return c;
 }
 
-// The 64 x 16 tiles of every lattice into dt, ordered by class and within a
-// class largest lattice first; records the class ranges and the classes, and
-// makes a branch stream for every class present after the first.
+using MultiTile = lbm::MultiLarge<LBM_F32>;
+static_assert(MultiTile::TX == lbm::MultiLarge<LBM_F16DEV>::TX && MultiTile::TY == lbm::MultiLarge<LBM_F16DEV>::TY,
+              "one multi-step tile shape for every storage kind");
+
+// Tiles of a lattice in the two-step or the multi-step tile shape.
+void tiles2_of(const lbm_s* h, bool multi, int* tx, int* ty) {
+    const int TX = multi ? MultiTile::TX : lbm::kBatchFusedTX, TY = multi ? MultiTile::TY : lbm::kBatchFusedTY;
+    *tx = (h->a.nx + TX - 1) / TX;
+    *ty = (h->a.ny + TY - 1) / TY;
+}
+
+bool multi_admitted(const lbm_batch_s* b) {
+    if (b->model != LBM_CASCADED) return false;
+    for (const lbm_s* h : b->doms)
+        if (lbm::force_mode(h) != 0 || h->a.rseed != 0) return false;
+    return true;
+}
+
+// The tiles of every lattice into dt, ordered by class and within a class
+// largest lattice first; records the tile shape, the class ranges and the
+// classes, and makes a branch stream for every class present after the first.
 cudaError_t order_tiles2(lbm_batch_s* b, int* dt) {
     const std::vector<int> cls = domain_classes(b);
+    const bool multi = multi_admitted(b);
     std::vector<int> idx(b->doms.size());
     std::iota(idx.begin(), idx.end(), 0);
     auto nodes = [&](int d) { return (long long)b->doms[d]->a.nx * b->doms[d]->a.ny; };
@@ -287,8 +314,8 @@ cudaError_t order_tiles2(lbm_batch_s* b, int* dt) {
     std::vector<int> t;
     int first[lbm::kBatchClasses + 1] = {};
     for (int d : idx) {
-        const int tx = (b->doms[d]->a.nx + lbm::kBatchFusedTX - 1) / lbm::kBatchFusedTX;
-        const int ty = (b->doms[d]->a.ny + lbm::kBatchFusedTY - 1) / lbm::kBatchFusedTY;
+        int tx, ty;
+        tiles2_of(b->doms[d], multi, &tx, &ty);
         for (int j = 0; j < ty; ++j)
             for (int i = 0; i < tx; ++i) t.insert(t.end(), {d, i, j});
         first[cls[d] + 1] += tx * ty;
@@ -316,20 +343,25 @@ cudaError_t order_tiles2(lbm_batch_s* b, int* dt) {
     if (e != cudaSuccess) return e;
     std::copy(first, first + lbm::kBatchClasses + 1, b->class_first);
     b->cls2 = cls;
+    b->multi = multi;
+    b->ntiles2 = int(t.size() / 3);
     return cudaSuccess;
 }
 
-// Second arrays and tensor maps of every lattice, the 64 x 16 tile list and
-// the error word; made once.
+// Second arrays and tensor maps of every lattice, the tile list (room for
+// either tile shape) and the error word; made once.
 cudaError_t prepare_two_step(lbm_batch_s* b) {
     if (b->h_pairs) return cudaSuccess;
     cudaError_t e = cudaSuccess;
     for (lbm_s* h : b->doms)
         if (e == cudaSuccess) e = lbm_prepare_two_step(h);
     size_t ntiles = 0;  // fewer than the one-step list's, whose size lbm_batch_create bounds
-    for (const lbm_s* h : b->doms)
-        ntiles += size_t((h->a.nx + lbm::kBatchFusedTX - 1) / lbm::kBatchFusedTX) *
-                  ((h->a.ny + lbm::kBatchFusedTY - 1) / lbm::kBatchFusedTY);
+    for (const lbm_s* h : b->doms) {
+        int tx, ty, mx, my;
+        tiles2_of(h, false, &tx, &ty);
+        tiles2_of(h, true, &mx, &my);
+        ntiles += std::max(size_t(tx) * ty, size_t(mx) * my);
+    }
     lbm::BatchPair* hp = nullptr;
     lbm::BatchPair* dp = nullptr;
     int* dt = nullptr;
@@ -347,7 +379,6 @@ cudaError_t prepare_two_step(lbm_batch_s* b) {
         if (de) cudaFree(de);
         return e;
     }
-    b->ntiles2 = int(ntiles);
     b->h_pairs = hp;
     b->d_pairs = dp;
     b->d_tiles2 = dt;
@@ -355,9 +386,11 @@ cudaError_t prepare_two_step(lbm_batch_s* b) {
     return cudaSuccess;
 }
 
-cudaError_t launch_class(lbm_batch_s* b, int c, int k, int rstride, int kstep, cudaStream_t s) {
+cudaError_t launch_class(lbm_batch_s* b, int c, int k, int rstride, int kstep, int steps, cudaStream_t s) {
     const int n = b->class_first[c + 1] - b->class_first[c];
     const int* tiles = b->d_tiles2 + 3 * b->class_first[c];
+    if (b->multi)
+        return lbm::launch_batch_multi_cascaded(lbm::class_store(c), n, b->d_doms, b->d_pairs, tiles, k, steps, b->d_err, s);
     switch (b->model) {
         case LBM_CASCADED:
             return lbm::launch_batch_fused_cascaded(c, n, b->d_doms, b->d_pairs, tiles, k, b->d_rtab, rstride, kstep,
@@ -371,12 +404,12 @@ cudaError_t launch_class(lbm_batch_s* b, int c, int k, int rstride, int kstep, c
     }
 }
 
-// Two-step launch k of a sequence (reads each lattice's arr[k & 1]); the round
-// table holds rstride hashes per lattice, two per launch from 2 kstep.  One
+// Launch k of a sequence (reads each lattice's arr[k & 1]) of `steps` steps, two
+// unless b->multi; the round table holds rstride hashes per lattice, two per launch from 2 kstep.  One
 // kernel per class present: the first on the batch stream, each other one on a
 // branch stream that waits for the batch stream and that the batch stream then
 // waits for, so the kernels run side by side (also inside a captured graph).
-cudaError_t launch_pair(lbm_batch_s* b, int k, int rstride, int kstep) {
+cudaError_t launch_pair(lbm_batch_s* b, int k, int rstride, int kstep, int steps) {
     int used[lbm::kBatchClasses];
     int n = 0;
     for (int c = 0; c < lbm::kBatchClasses; ++c)
@@ -385,21 +418,25 @@ cudaError_t launch_pair(lbm_batch_s* b, int k, int rstride, int kstep) {
     cudaError_t e = n > 1 ? cudaEventRecord(b->fork, b->stream) : cudaSuccess;
     for (int i = 0; i < n && e == cudaSuccess; ++i) {
         if (i == 0) {
-            e = launch_class(b, used[0], k, rstride, kstep, b->stream);
+            e = launch_class(b, used[0], k, rstride, kstep, steps, b->stream);
             continue;
         }
         const lbm_batch_s::Branch& br = b->branch[i - 1];
         e = cudaStreamWaitEvent(br.s, b->fork, 0);
-        if (e == cudaSuccess) e = launch_class(b, used[i], k, rstride, kstep, br.s);
+        if (e == cudaSuccess) e = launch_class(b, used[i], k, rstride, kstep, steps, br.s);
         if (e == cudaSuccess) e = cudaEventRecord(br.joined, br.s);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, br.joined, 0);
     }
     return e;
 }
 
-// Launches per replay of the two-step graph: graph_steps / 2, rounded down to an
-// even number (the arrays are back in place after each replay).
-int pair_graph_len(const lbm_batch_s* b) { return (b->graph_steps / 4) * 2; }
+// Steps of a full launch.
+int launch_steps(const lbm_batch_s* b) { return b->multi ? lbm::kMultiSteps : 2; }
+
+// Launches per replay of the graph of full launches: graph_steps over the steps
+// of one, rounded down to an even number (the arrays are back in place after each
+// replay).
+int pair_graph_len(const lbm_batch_s* b) { return b->graph_steps / (2 * launch_steps(b)) * 2; }
 
 cudaError_t build_graph2(lbm_batch_s* b) {
     if (b->graph2) cudaGraphExecDestroy(b->graph2);
@@ -408,7 +445,7 @@ cudaError_t build_graph2(lbm_batch_s* b) {
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
-    for (int k = 0; k < len && e == cudaSuccess; ++k) e = launch_pair(b, k & 1, 2 * len, k);
+    for (int k = 0; k < len && e == cudaSuccess; ++k) e = launch_pair(b, k & 1, 2 * len, k, launch_steps(b));
     cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
     if (e == cudaSuccess) e = e2;
     if (e == cudaSuccess) e = cudaGraphInstantiate(&b->graph2, g, 0);
@@ -416,24 +453,29 @@ cudaError_t build_graph2(lbm_batch_s* b) {
     return e;
 }
 
-// `pairs` two-step launches from the domains' current steps plus `base` (all
-// even); the lattices' arrays trade roles if pairs is odd.
+// `pairs` pairs of steps from the domains' current steps plus `base` (all even),
+// in full launches and a two-step one for the rest; the lattices' arrays trade
+// roles if the number of launches is odd.
 cudaError_t run_pairs(lbm_batch_s* b, long pairs, long long base) {
     cudaError_t e = cudaSuccess;
-    long p = 0;
+    const long full = launch_steps(b) / 2;  // pairs of a full launch
+    long p = 0, launches = 0;
     const int len = pair_graph_len(b);
-    if (len > 0 && pairs >= len) {
+    if (len > 0 && pairs >= len * full) {
         if (!b->graph2) e = build_graph2(b);
-        for (; e == cudaSuccess && pairs - p >= len; p += len) {
+        for (; e == cudaSuccess && pairs - p >= len * full; p += len * full) {
             e = fill_round_table(b, 2 * len, base + 2 * p);
             if (e == cudaSuccess) e = cudaGraphLaunch(b->graph2, b->stream);
         }
     }
-    for (; e == cudaSuccess && p < pairs; ++p) {
+    while (e == cudaSuccess && p < pairs) {
+        const long take = pairs - p >= full ? full : 1;
         e = fill_round_table(b, 2, base + 2 * p);
-        if (e == cudaSuccess) e = launch_pair(b, int(p & 1), 2, 0);
+        if (e == cudaSuccess) e = launch_pair(b, int(launches & 1), 2, 0, int(2 * take));
+        p += take;
+        ++launches;
     }
-    if (e == cudaSuccess && (pairs & 1)) {
+    if (e == cudaSuccess && (launches & 1)) {
         for (lbm_s* h : b->doms) {
             std::swap(h->state, h->state_alt);
             h->a.f = h->state;
@@ -747,15 +789,15 @@ int lbm_batch_tune(lbm_batch_t b, int trial_steps, float* best_ms) {
             if (e == cudaSuccess) e = cudaEventRecord(b->done, b->stream);
             if (e == cudaSuccess) e = refresh_domains(b);
             if (e == cudaSuccess) e = fill_round_table(b, 2, 0);
-            for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = launch_pair(b, k & 1, 2, 0);
+            for (int k = 0; k < 2 && e == cudaSuccess; ++k) e = launch_pair(b, k & 1, 2, 0, launch_steps(b));
             if (e == cudaSuccess) e = cudaEventRecord(t0, b->stream);
-            for (int k = 0; k < launches && e == cudaSuccess; ++k) e = launch_pair(b, k & 1, 2, 0);
+            for (int k = 0; k < launches && e == cudaSuccess; ++k) e = launch_pair(b, k & 1, 2, 0, launch_steps(b));
             if (e == cudaSuccess) e = cudaEventRecord(t1, b->stream);
             if (e == cudaSuccess) e = cudaEventSynchronize(t1);
             float ms = 0.f;
             if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, t0, t1);
-            if (e == cudaSuccess && ms / (2 * launches) < best_step) {
-                best_step = ms / (2 * launches);
+            if (e == cudaSuccess && ms / (launch_steps(b) * launches) < best_step) {
+                best_step = ms / (launch_steps(b) * launches);
                 best_two = true;
             }
             if (e == cudaSuccess) e = copy_all(false);
@@ -785,8 +827,8 @@ int lbm_batch_tune(lbm_batch_t b, int trial_steps, float* best_ms) {
 int lbm_batch_info(lbm_batch_t b, int cfg[6], void** stream) {
     if (!b) return fail(LBM_EINVAL, "null batch");
     if (cfg && b->two_step) {
-        cfg[0] = lbm::kBatchFusedTX;
-        cfg[1] = lbm::kBatchFusedTY;
+        cfg[0] = b->multi ? MultiTile::TX : lbm::kBatchFusedTX;
+        cfg[1] = b->multi ? MultiTile::TY : lbm::kBatchFusedTY;
         cfg[2] = 4;
         cfg[3] = 0;
         cfg[4] = b->ntiles2;

@@ -1,4 +1,4 @@
-// lbm_batch_cascaded.cu -- batch kernels (one step, and two steps per launch) for the cascaded collision.
+// lbm_batch_cascaded.cu -- batch kernels (one step, and several steps per launch) for the cascaded collision.
 #include "lbm_batch_fused.cuh"
 #include "lbm_batch_impl.cuh"
 
@@ -18,5 +18,13 @@ cudaError_t launch_batch_fused_cascaded(int cls, int ntiles, const BatchDomain* 
                                   const int* tiles, int k, const unsigned* rtab, int rstride, int kstep, int* err,
                                   cudaStream_t s) {
     return launch_batch_fused_model<LBM_CASCADED>(cls, ntiles, doms, pairs, tiles, k, rtab, rstride, kstep, err, s);
+}
+cudaError_t launch_batch_multi_cascaded(int store, int ntiles, const BatchDomain* doms, const BatchPair* pairs,
+                                        const int* tiles, int k, int steps, int* err, cudaStream_t s) {
+    switch (store) {
+        case LBM_F32: return launch_batch_multi<LBM_F32>(ntiles, doms, pairs, tiles, k, steps, err, s);
+        case LBM_F16DEV: return launch_batch_multi<LBM_F16DEV>(ntiles, doms, pairs, tiles, k, steps, err, s);
+        default: return launch_batch_multi<LBM_BF16DEV>(ntiles, doms, pairs, tiles, k, steps, err, s);
+    }
 }
 }  // namespace lbm

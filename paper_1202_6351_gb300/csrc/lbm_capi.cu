@@ -227,7 +227,7 @@ cudaError_t launch_fused_at(lbm_s* h, long t, long left, int* took) {
     cudaError_t e;
     if (multi_active(h)) {
         *took = left >= lbm::kMultiSteps ? lbm::kMultiSteps : 2;
-        const CUtensorMap& map = h->mmap[h->tmap_ptr[0] == a.f ? 0 : 1];
+        const CUtensorMap& map = lbm_multi_map(h, a.f);
         switch (h->store) {
             case LBM_F32: e = lbm::launch_multi_f32(map, a, h->state_alt, h->d_err, *took, h->stream); break;
             case LBM_BF16DEV: e = lbm::launch_multi_bf16(map, a, h->state_alt, h->d_err, *took, h->stream); break;
@@ -404,6 +404,7 @@ int after_reset(lbm_s* h) {
 
 cudaError_t lbm_prepare_two_step(lbm_s* h) { return ensure_fused(h); }
 const CUtensorMap& lbm_tensor_map(const lbm_s* h, const void* base) { return map_of(h, base); }
+const CUtensorMap& lbm_multi_map(const lbm_s* h, const void* base) { return h->mmap[h->tmap_ptr[0] == base ? 0 : 1]; }
 
 extern "C" {
 

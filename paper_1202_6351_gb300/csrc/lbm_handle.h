@@ -50,3 +50,5 @@ cudaError_t lbm_prepare_two_step(lbm_s* h);
 // The tensor map of population array `base` (h->state or h->state_alt) after
 // lbm_prepare_two_step.
 const CUtensorMap& lbm_tensor_map(const lbm_s* h, const void* base);
+// The same with the box of the multi-step kernel.
+const CUtensorMap& lbm_multi_map(const lbm_s* h, const void* base);

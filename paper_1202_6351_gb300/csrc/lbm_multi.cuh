@@ -295,21 +295,18 @@ __device__ __forceinline__ void multi_load_cells(const Args& a, const typename G
 }
 
 // `steps` (2 or 4) steps of one tile from `in` (natural layout, even step) into `out`.
+// smem holds G::SMEM bytes (1024-byte aligned); bar and ok live in shared memory
+// and serve this tile only.  Every thread of the CTA calls this alike.
 template <class G>
-__global__ void __launch_bounds__(G::NT, G::MINB)
-    multi_kernel(const __grid_constant__ CUtensorMap map, const Args a, const void* __restrict__ in, void* __restrict__ out,
-                 int* __restrict__ err, int steps) {
+__device__ __forceinline__ void multi_tile(const CUtensorMap* map, const Args& a, const void* in, void* out, int* err, int x0,
+                                           int y0, int steps, unsigned char* smem, unsigned long long* bar, int* ok) {
     using T = typename G::T;
-    extern __shared__ __align__(1024) unsigned char multi_smem[];
-    __shared__ __align__(8) unsigned long long bar;
-    __shared__ int ok;
-    T* A = reinterpret_cast<T*>(multi_smem);
-    const int tid = threadIdx.x, x0 = blockIdx.x * G::TX, y0 = blockIdx.y * G::TY;
+    T* A = reinterpret_cast<T*>(smem);
+    const int tid = threadIdx.x;
     const bool perx = !a.wall[LBM_WEST], pery = !a.wall[LBM_SOUTH];
     const T* f = static_cast<const T*>(in);
-    pdl_wait();
     if constexpr (G::TMA) {
-        if (!multi_load_tma<G>(&map, a, f, A, err, x0, y0, steps, &bar, &ok)) return;
+        if (!multi_load_tma<G>(map, a, f, A, err, x0, y0, steps, bar, ok)) return;
     } else {
         multi_load_cells<G>(a, f, A, x0, y0, steps);
     }
@@ -352,6 +349,17 @@ __global__ void __launch_bounds__(G::NT, G::MINB)
             for (int q = 0; q < 9; ++q) dst[q * a.plane] = p[q * G::PLANE];
         }
     }
+}
+
+template <class G>
+__global__ void __launch_bounds__(G::NT, G::MINB)
+    multi_kernel(const __grid_constant__ CUtensorMap map, const Args a, const void* __restrict__ in, void* __restrict__ out,
+                 int* __restrict__ err, int steps) {
+    extern __shared__ __align__(1024) unsigned char multi_smem[];
+    __shared__ __align__(8) unsigned long long bar;
+    __shared__ int ok;
+    pdl_wait();
+    multi_tile<G>(&map, a, in, out, err, blockIdx.x * G::TX, blockIdx.y * G::TY, steps, multi_smem, &bar, &ok);
 }
 
 template <class G>

@@ -48,3 +48,37 @@ def test_multi_step_launches_are_bitwise_equal_to_single_steps(shape, edges, sto
             assert L.time == 24
     for a, b in zip(states[0], states[3]):
         np.testing.assert_array_equal(a, b)
+
+
+@pytest.mark.parametrize("start", [0, 1], ids=["even_start", "odd_start"])
+def test_batches_of_unforced_lattices_take_four_steps_per_launch(start):
+    """A batch whose lattices all take the multi-step tile, against the lattices
+    stepped alone; a force set on one lattice between calls moves the batch to the
+    two-step tiles and its removal back."""
+    om = (1.1, 1.7, 1.7, 1.0, 1.2, 0.9)
+    specs = [(64, 64, lbm.F32, "periodic"), (57, 41, lbm.F16DEV, "cavity"), (113, 37, lbm.F32, "channel_x"),
+             (4, 5, lbm.BF16DEV, "periodic"), (300, 7, lbm.F16DEV, "channel_y"), (56, 80, lbm.F32, "cavity")]
+
+    def make(i):
+        nx, ny, store, edges = specs[i]
+        L = lbm.Lattice(nx, ny, om, edges=EDGES[edges][0], wall_u=EDGES[edges][1], store=store)
+        return L.init(*workloads.random_fields(i, nx, ny, u_amp=0.03, rho_amp=0.01)).step(start)
+
+    alone, batched = ([make(i) for i in range(len(specs))] for _ in range(2))
+    with lbm.Batch(batched) as B:
+        B.set_graph_steps(20)  # two launches of four steps, twice per replay
+        B.set_two_step(True)
+        for force, tile in (((0.0, 0.0), (56, 40)), ((1e-5, 0.0), (64, 16)), ((0.0, 0.0), (56, 40))):
+            for L in (alone[0], batched[0]):
+                L.set_force(force)
+            for n in (29, 6, 2):
+                B.step(n)
+                for L in alone:
+                    L.step(n)
+            assert B.info()["tile"] == tile
+            B.sync()
+            for i, (a, b) in enumerate(zip(alone, batched)):
+                assert a.time == b.time
+                np.testing.assert_array_equal(a.get_f(), b.get_f(), err_msg=f"lattice {i}")
+    for L in alone + batched:
+        L.close()
