@@ -17,18 +17,37 @@ using lbm3::Args3;
 
 namespace {
 
-constexpr int kBX = 128, kBY = 2;
+constexpr int kBX = 128, kBY = 2;  // blocks of the initialisation and transfer kernels
 
+constexpr int kStep3Threads = 128;
+
+// One step, one node per thread.  A block takes 2^lbx columns of
+// kStep3Threads / 2^lbx node rows, rows (y, z) numbered through, nbx blocks to a
+// row: a row of 192 nodes in 128-wide blocks leaves a quarter of the lanes idle,
+// rows that do not fill a block in y idle warps.
+// FP32 storage is bound by HBM and load latency (216 B per update, 83 % of copy
+// bandwidth on 192^3), 16-bit storage by instruction issue: 758 instructions per
+// node on the even step and 920 on the odd one, 620 of them the collision; with
+// 64-bit slot offsets per population they were 873 and 1148.  The 27 slots of a
+// node are nine row and three column offsets, kept in registers from load to
+// store: five blocks per SM (96 registers; FP32 192^3 us per step with four, five,
+// six, seven: 283, 271, 282, 321).
+// us per step, before -> now: FP32 192^3 327 -> 271, 128^3 91.1 -> 81.9, FP16 128^3
+// 81.8 -> 69.7, 127 x 96 x 130 60.5 -> 51.6, FP32 40 x 33 x 27 6.2 -> 3.0.
 template <int STORE, bool ODD, bool FORCED>
-__global__ void __launch_bounds__(kBX * kBY) step3_kernel(const Args3 a) {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    if (x >= a.nx || y >= a.ny) return;
+__global__ void __launch_bounds__(kStep3Threads, STORE == LBM_F64 ? 1 : 5) step3_kernel(const Args3 a, int lbx, unsigned nbx) {
+    const unsigned rb = blockIdx.x / nbx, cb = blockIdx.x - rb * nbx;
+    const int x = int(cb << lbx) + int(threadIdx.x & ((1u << lbx) - 1u));
+    const unsigned row = rb * (kStep3Threads >> lbx) + (threadIdx.x >> lbx);
+    const unsigned z = row / unsigned(a.ny);
+    const int y = int(row - z * unsigned(a.ny));
+    lbm::pdl_wait();
+    if (x >= a.nx || z >= unsigned(a.nz)) return;
     typename lbm::Store<STORE>::R d[27];
-    lbm3::load3<STORE, ODD>(a, x, y, z, d);
+    const lbm3::Slots3 s = lbm3::slots3<ODD>(a, x, y, int(z));
+    lbm3::load3<STORE, ODD>(a, s, d);
     lbm3::collide3<typename lbm::Store<STORE>::R, FORCED>(d, a);
-    lbm3::store3<STORE, ODD>(a, x, y, z, d);
+    lbm3::store3<STORE, ODD>(a, s, d);
 }
 
 // rho [nz][ny][nx], u [3][nz][ny][nx] (FP64, device; either may be null: rho0 / rest)
@@ -49,7 +68,7 @@ __global__ void __launch_bounds__(kBX * kBY) init3_kernel(const Args3 a, const d
     R d[27];
     lbm3::equilibrium3<R>(d, rho0, drho, ux, uy, uz, k[lbm3::K3_FX], k[lbm3::K3_FY], k[lbm3::K3_FZ]);
     T* f = static_cast<T*>(a.f);
-    const long long o = lbm3::node_off<T>(a, x, y, z);
+    const int o = lbm3::node_off<T>(a, x, y, z);
 #pragma unroll
     for (int q = 0; q < 27; ++q) f[q * a.plane + o] = S::enc(d[q]);
 }
@@ -82,7 +101,7 @@ __global__ void __launch_bounds__(kBX * kBY) set3_kernel(const Args3 a, const do
     if (x >= a.nx || y >= a.ny) return;
     const long long p = ((long long)z * a.ny + y) * a.nx + x, n = (long long)a.nx * a.ny * a.nz;
     T* f = static_cast<T*>(a.f);
-    const long long o = lbm3::node_off<T>(a, x, y, z);
+    const int o = lbm3::node_off<T>(a, x, y, z);
 #pragma unroll
     for (int q = 0; q < 27; ++q)
         f[q * a.plane + o] = S::enc(typename S::R((in[q * n + p] - lbm3::wgt<double>(q) * a.kd[lbm3::K3_RHO0]) * a.scale));
@@ -125,15 +144,19 @@ dim3 grid_of(const Args3& a) { return dim3((a.nx + kBX - 1) / kBX, (a.ny + kBY -
 
 template <int STORE>
 cudaError_t launch_step3(const Args3& a, bool odd, bool forced, cudaStream_t s) {
-    const dim3 g = grid_of(a), b(kBX, kBY);
-    if (odd) {
-        if (forced) step3_kernel<STORE, true, true><<<g, b, 0, s>>>(a);
-        else step3_kernel<STORE, true, false><<<g, b, 0, s>>>(a);
-    } else {
-        if (forced) step3_kernel<STORE, false, true><<<g, b, 0, s>>>(a);
-        else step3_kernel<STORE, false, false><<<g, b, 0, s>>>(a);
-    }
-    return cudaGetLastError();
+    // The block width with the fewest idle lanes in a row, the widest of equals.
+    int lbx = 7;
+    auto padded = [&](int l) { return (a.nx + (1 << l) - 1) >> l << l; };
+    for (int l = 6; l >= 5; --l)
+        if (padded(l) < padded(lbx)) lbx = l;
+    const unsigned nbx = unsigned(padded(lbx)) >> lbx;
+    const unsigned rows = unsigned(a.ny) * unsigned(a.nz), per = unsigned(kStep3Threads) >> lbx;
+    const dim3 g(nbx * ((rows + per - 1) / per)), b(kStep3Threads);
+    if (odd)
+        return forced ? lbm::launch_chain(step3_kernel<STORE, true, true>, g, b, 0, s, a, lbx, nbx)
+                      : lbm::launch_chain(step3_kernel<STORE, true, false>, g, b, 0, s, a, lbx, nbx);
+    return forced ? lbm::launch_chain(step3_kernel<STORE, false, true>, g, b, 0, s, a, lbx, nbx)
+                  : lbm::launch_chain(step3_kernel<STORE, false, false>, g, b, 0, s, a, lbx, nbx);
 }
 
 int fail(int code, const char* msg) { return lbm::set_error(code, "%s", msg); }

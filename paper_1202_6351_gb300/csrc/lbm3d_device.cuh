@@ -209,47 +209,66 @@ __device__ __forceinline__ void equilibrium3(R d[27], R rho0, R drho, R ux, R uy
 // even step: node x reads slot a of x and writes post-collision a into slot
 // opp(a) of x; odd step: node x reads slot opp(a) of x - e_a and writes
 // post-collision a into slot a of x + e_a.
+// Offsets inside one plane are 32-bit (pitch * ny * nz < 2^31 is checked at
+// creation); the plane base f + q * plane is the same for every thread.
 template <typename T>
-__device__ __forceinline__ long long node_off(const Args3& a, int x, int y, int z) {
-    return ((long long)z * a.ny + y) * a.pitch + x;
+__device__ __forceinline__ int node_off(const Args3& a, int x, int y, int z) {
+    return (z * a.ny + y) * a.pitch + x;
 }
 
+// Slots of node (x, y, z): `own`, and on odd steps the neighbour's at x + s e_a
+// as the sum of a row offset (y, z) and a column.
+struct Slots3 {
+    int row[9], col[3];  // row[(e_y + 1) + 3 (e_z + 1)], col[e_x + 1]
+};
+template <bool ODD>
+__device__ __forceinline__ Slots3 slots3(const Args3& a, int x, int y, int z) {
+    Slots3 s;
+    const int ym = y > 0 ? y - 1 : a.ny - 1, yp = y < a.ny - 1 ? y + 1 : 0;
+    const int zm = z > 0 ? z - 1 : a.nz - 1, zp = z < a.nz - 1 ? z + 1 : 0;
+    const int ys[3] = {ym, y, yp}, zs[3] = {zm, z, zp};
+    if (ODD) {
+#pragma unroll
+        for (int k = 0; k < 9; ++k) s.row[k] = (zs[k / 3] * a.ny + ys[k % 3]) * a.pitch;
+        s.col[0] = x > 0 ? x - 1 : a.nx - 1;
+        s.col[1] = x;
+        s.col[2] = x < a.nx - 1 ? x + 1 : 0;
+    } else {
+        s.row[4] = (z * a.ny + y) * a.pitch;
+        s.col[1] = x;
+    }
+    return s;
+}
+// offset of the slot at x + e_q
+template <bool ODD>
+__device__ __forceinline__ int slot3(const Slots3& s, int q) {
+    if (!ODD) return s.row[4] + s.col[1];
+    return s.row[(ey(q) + 1) + 3 * (ez(q) + 1)] + s.col[ex(q) + 1];
+}
+
+// Loads and stores of a step go to the same 27 slots: plane p at x + e_p on odd
+// steps (population opp(p) is read there and population p written), plane p at x on
+// even ones (p is read, opp(p) written).
 template <int STORE, bool ODD>
-__device__ __forceinline__ void load3(const Args3& a, int x, int y, int z, typename lbm::Store<STORE>::R d[27]) {
+__device__ __forceinline__ void load3(const Args3& a, const Slots3& s, typename lbm::Store<STORE>::R d[27]) {
     using S = lbm::Store<STORE>;
     using T = typename S::T;
     const T* __restrict__ f = static_cast<const T*>(a.f);
-    if (!ODD) {
-        const long long n = node_off<T>(a, x, y, z);
 #pragma unroll
-        for (int q = 0; q < 27; ++q) d[q] = S::dec(f[q * a.plane + n]);
-    } else {
-        const int xs[3] = {x > 0 ? x - 1 : a.nx - 1, x, x < a.nx - 1 ? x + 1 : 0};
-        const int ys[3] = {y > 0 ? y - 1 : a.ny - 1, y, y < a.ny - 1 ? y + 1 : 0};
-        const int zs[3] = {z > 0 ? z - 1 : a.nz - 1, z, z < a.nz - 1 ? z + 1 : 0};
-#pragma unroll
-        for (int q = 0; q < 27; ++q)  // source x - e_q: index 1 - e
-            d[q] = S::dec(f[opp(q) * a.plane + node_off<T>(a, xs[1 - ex(q)], ys[1 - ey(q)], zs[1 - ez(q)])]);
-    }
+    for (int p = 0; p < 27; ++p) d[ODD ? opp(p) : p] = S::dec((f + p * a.plane)[slot3<ODD>(s, p)]);
+}
+template <int STORE, bool ODD>
+__device__ __forceinline__ void load3(const Args3& a, int x, int y, int z, typename lbm::Store<STORE>::R d[27]) {
+    load3<STORE, ODD>(a, slots3<ODD>(a, x, y, z), d);
 }
 
 template <int STORE, bool ODD>
-__device__ __forceinline__ void store3(const Args3& a, int x, int y, int z, const typename lbm::Store<STORE>::R d[27]) {
+__device__ __forceinline__ void store3(const Args3& a, const Slots3& s, const typename lbm::Store<STORE>::R d[27]) {
     using S = lbm::Store<STORE>;
     using T = typename S::T;
     T* __restrict__ f = static_cast<T*>(a.f);
-    if (!ODD) {
-        const long long n = node_off<T>(a, x, y, z);
 #pragma unroll
-        for (int q = 0; q < 27; ++q) f[opp(q) * a.plane + n] = S::enc(d[q]);
-    } else {
-        const int xs[3] = {x > 0 ? x - 1 : a.nx - 1, x, x < a.nx - 1 ? x + 1 : 0};
-        const int ys[3] = {y > 0 ? y - 1 : a.ny - 1, y, y < a.ny - 1 ? y + 1 : 0};
-        const int zs[3] = {z > 0 ? z - 1 : a.nz - 1, z, z < a.nz - 1 ? z + 1 : 0};
-#pragma unroll
-        for (int q = 0; q < 27; ++q)  // target x + e_q: index 1 + e
-            f[q * a.plane + node_off<T>(a, xs[1 + ex(q)], ys[1 + ey(q)], zs[1 + ez(q)])] = S::enc(d[q]);
-    }
+    for (int p = 0; p < 27; ++p) (f + p * a.plane)[slot3<ODD>(s, p)] = S::enc(d[ODD ? p : opp(p)]);
 }
 
 }  // namespace lbm3
