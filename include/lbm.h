@@ -185,12 +185,17 @@ int lbm_init(lbm_t h, const double* rho, const double* u);
 int lbm_init_device(lbm_t h, const double* rho, const double* u);
 
 /* Advance n >= 0 time steps (collide Eq. 23 + stream Eq. 24 per step), one
- * fused kernel launch per step, asynchronously on the handle's stream.  Runs
+ * fused kernel launch per step (several with variant 3), asynchronously on the
+ * handle's stream.  Small lattices (LBM_F32, LBM_BF16DEV, LBM_F16DEV; up to
+ * 16 x 800 nodes, with a sixteenth of the rows, rounded up, of at most 800 nodes;
+ * every variant but 1) take 8 or more steps in one launch of a kernel that keeps
+ * the lattice in the shared memory of one thread-block cluster; the results are
+ * bit for bit those of variants 0, 2 and 3.  Elsewhere runs
  * of at least lbm_set_graph_steps steps starting at an even step are replayed
  * from a CUDA graph on an internal stream that is ordered after the handle's
  * stream and before any later work on it (the graph is recaptured whenever a
  * rate, force, force field, variant or rounding mode has changed).  With the divergence
- * check on (lbm_set_check) no graph is used, the call synchronises at every
+ * check on (lbm_set_check) the call synchronises at every
  * check and returns LBM_EDIVERGED when it fails. */
 int lbm_step(lbm_t h, long n);
 

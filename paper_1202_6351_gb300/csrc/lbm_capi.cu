@@ -14,6 +14,7 @@
 #include "lbm_fused.cuh"
 #include "lbm_internal.h"
 #include "lbm_multi.cuh"
+#include "lbm_resident.cuh"
 #include "lbm_handle.h"
 
 using lbm::Args;
@@ -296,6 +297,27 @@ bool same_launch(const Args& x, const Args& y) {
     for (int k = 0; k < lbm::K_COUNT; ++k)
         if (x.kd[k] != y.kd[k] || x.kf[k] != y.kf[k]) return false;
     return true;
+}
+
+// Steps h->t .. h->t + n - 1 by the small-lattice kernel.
+cudaError_t launch_resident(const lbm_s* h, int n) {
+    const unsigned long long t = static_cast<unsigned long long>(h->t);
+    switch (h->store) {
+        case LBM_F32: return lbm::launch_resident_f32(h->a, h->model, force_mode(h), t, n, h->stream);
+        case LBM_BF16DEV: return lbm::launch_resident_bf16(h->a, h->model, force_mode(h), t, n, h->stream);
+        default: return lbm::launch_resident_f16(h->a, h->model, force_mode(h), t, n, h->stream);
+    }
+}
+
+// Small FP32 and 16-bit lattices step on chip, whatever the variant (the results are
+// those of variants 0, 2 and 3); variant 1, which rounds differently, stays itself.
+bool resident_active(lbm_s* h) {
+    if (h->store == LBM_F64 || h->a.variant == 1 || !lbm::resident_fits(h->a)) return false;
+    if (h->resident < 0) {
+        h->resident = launch_resident(h, 0) == cudaSuccess ? 1 : 0;
+        if (!h->resident) cudaGetLastError();
+    }
+    return h->resident == 1;
 }
 
 void drop_graph(lbm_s* h) {
@@ -741,24 +763,25 @@ int lbm_step(lbm_t h, long n) {
     if (n < 0) return fail(LBM_EINVAL, "step count must be >= 0");
     const bool fused = fused_active(h);
     if (fused) LBM_CUDA(ensure_fused(h), "second population array for fused steps");
+    const bool resident = n >= lbm::kResidentMinSteps && resident_active(h);
     for (long s = 0; s < n;) {
+        // steps up to the end of the call or the next divergence check
+        const long left = h->check_every > 0 ? std::min(n - s, h->check_every - h->t % h->check_every) : n - s;
         const int len = graph_len(h);
-        if (len > 0 && h->check_every == 0 && (h->t & 1) == 0 && n - s >= len) {
+        int took = 1;
+        if (resident && left >= lbm::kResidentMinSteps) {
+            took = int(std::min(left, lbm::kResidentMaxSteps));
+            LBM_CUDA(launch_resident(h, took), "small-lattice steps");
+        } else if (len > 0 && (h->t & 1) == 0 && left >= len) {
+            took = len;
             LBM_CUDA(replay_graph(h), "step graph");
-            h->t += len;
-            s += len;
-            continue;
+        } else if (fused && (h->t & 1) == 0 && left >= 2) {
+            LBM_CUDA(launch_fused_at(h, h->t, left, &took), "fused step launch");
+        } else {
+            LBM_CUDA(launch_step(h, (h->t & 1) != 0), "step kernel launch");
         }
-        if (fused && (h->t & 1) == 0 && n - s >= 2) {
-            int took = 0;
-            LBM_CUDA(launch_fused_at(h, h->t, n - s, &took), "fused step launch");
-            h->t += took;
-            s += took;
-            continue;
-        }
-        LBM_CUDA(launch_step(h, (h->t & 1) != 0), "step kernel launch");
-        ++h->t;
-        ++s;
+        h->t += took;
+        s += took;
         if (h->check_every > 0 && h->t % h->check_every == 0) {
             double st[3];
             int rc = stats_into(h, st);

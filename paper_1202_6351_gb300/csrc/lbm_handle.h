@@ -42,6 +42,7 @@ struct lbm_s {
     CUtensorMap tmap[2], mmap[2];  // boxes of the two-step and of the multi-step kernel
     void* tmap_ptr[2] = {nullptr, nullptr};
     int* d_err = nullptr;
+    int resident = -1;           // whether the device can run the small-lattice kernel (-1: not asked yet)
 };
 
 // The second population array and the tensor maps of both arrays (variant 3),

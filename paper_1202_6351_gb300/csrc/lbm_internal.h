@@ -66,6 +66,12 @@ cudaError_t launch_multi_f32(const CUtensorMap& map, const Args& a, void* out, i
 cudaError_t launch_multi_bf16(const CUtensorMap& map, const Args& a, void* out, int* err, int steps, cudaStream_t s);
 cudaError_t launch_multi_f16(const CUtensorMap& map, const Args& a, void* out, int* err, int steps, cudaStream_t s);
 
+// Steps t0 .. t0 + n - 1 of a small lattice in one launch (lbm_resident.cuh); n = 0
+// only asks whether the device can run it.
+cudaError_t launch_resident_f32(const Args& a, int model, int force, unsigned long long t0, int n, cudaStream_t s);
+cudaError_t launch_resident_bf16(const Args& a, int model, int force, unsigned long long t0, int n, cudaStream_t s);
+cudaError_t launch_resident_f16(const Args& a, int model, int force, unsigned long long t0, int n, cudaStream_t s);
+
 // Auxiliary kernels (lbm_aux.cu); every field argument is dense [..][ny][nx] FP64 device memory.
 cudaError_t launch_init(const Args& a, int store, int model, int force, const double* rho, const double* u,
                         cudaStream_t s);
