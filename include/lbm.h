@@ -157,7 +157,7 @@ int lbm_set_variant(lbm_t h, int variant);
 int lbm_set_rounding(lbm_t h, int mode, unsigned long long seed);
 
 /* Autotuner for one lattice: times `trial_steps` steps of each kernel variant
- * the storage admits with each CTA shape (128x2, 256x1, 64x4, 32x8 threads;
+ * the storage admits with each CTA shape (128x1, 64x2, 32x4 threads;
  * variant 3 has fixed tiles) on the lattice itself (the state is snapshot
  * and restored, so it is left unchanged) and keeps the fastest pair; ms (may
  * be NULL) receives the best time per step of variants 0..3 (0 where not run).

@@ -616,7 +616,7 @@ int lbm_tune(lbm_t h, int trial_steps, float ms[LBM_NUM_VARIANTS]) {
     const int steps = trial_steps + (trial_steps & 1);  // even: the state returns to its layout
     if (ms)
         for (int v = 0; v < LBM_NUM_VARIANTS; ++v) ms[v] = 0.f;
-    static const int widths[4] = {128, 256, 64, 32};  // CTA shapes 128x2, 256x1, 64x4, 32x8
+    static const int widths[3] = {128, 64, 32};  // CTA shapes 128x1, 64x2, 32x4
     const int v_prev = h->a.variant;
     // `steps` steps from step h->t as lbm_step takes them without graphs
     auto run = [&](int k0, int count) -> cudaError_t {
@@ -648,7 +648,7 @@ int lbm_tune(lbm_t h, int trial_steps, float ms[LBM_NUM_VARIANTS]) {
             continue;
         }
         float best_of_v = 1e30f;
-        for (int wi = 0; wi < (v == 3 ? 1 : 4) && e == cudaSuccess; ++wi) {  // variant 3 has a fixed tile
+        for (int wi = 0; wi < (v == 3 ? 1 : 3) && e == cudaSuccess; ++wi) {  // variant 3 has a fixed tile
             h->a.variant = v;
             h->a.block_x = widths[wi];
             e = run(0, 2);

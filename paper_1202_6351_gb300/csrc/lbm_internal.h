@@ -42,8 +42,12 @@ int force_mode(const lbm_s* h);
 cudaError_t launch_step_any(const Args& a, int store, int model, bool odd, int force, bool walls, cudaStream_t s);
 
 // Launch shape of the fused step kernel: one thread per node, BX x BY threads.
+// Blocks of 128 threads rather than 256 leave a shorter last wave and spread more
+// evenly: FP32 us per step 512^2 3.17 -> 3.13, cavity 512^2 3.55 -> 3.38, 257^2 1.92 ->
+// 1.70, 1025^2 9.35 -> 9.09, 4096^2 189.6 -> 184.1 (384^2 2.15 -> 2.21); 64 threads are
+// slower from 384^2 to 1025^2.
 constexpr int kStepBX = 128;
-constexpr int kStepBY = 2;
+constexpr int kStepBY = 1;
 
 // One fused collide-and-stream step (defined once per storage type).
 cudaError_t launch_step_f64(const Args& a, int model, bool odd, int force, bool walls, cudaStream_t s);

@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(kStepBX * kStepBY) step_kernel_oop(const Args 
 // Two rows per thread (nodes (x, y) and (x, y + 1)) with packed FP32x2
 // arithmetic; a pair that touches a wall edge takes the per-node wall path.
 template <int MODEL, int STORE, bool ODD, int FORCE, bool WALLS>
-__global__ void __launch_bounds__(kStepBX * kStepBY, 4) step_kernel_pair(const Args a) {
+__global__ void __launch_bounds__(kStepBX * kStepBY, 8) step_kernel_pair(const Args a) {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = 2 * (blockIdx.y * blockDim.y + threadIdx.y);
     pdl_wait();
