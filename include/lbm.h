@@ -267,11 +267,23 @@ size_t lbm_bytes_per_update(int store);
  * state is copied; every = 1 keeps every state and recomputes nothing.
  * Device memory used during the call: (ceil(nsteps/every) +
  * max(1, min(every, nsteps) - 1)) times the population array, two adjoint
- * arrays, a segment force-gradient array (FP32 storage) and small scratch,
- * allocated and released in stream order.  Synchronous.
+ * arrays, a force-gradient array, its FP32 segment sum (FP32 storage) and small
+ * scratch, allocated and released in stream order.  Synchronous.
  * Leaves the lattice at step nsteps. */
 int lbm_adjoint_run(lbm_t h, long nsteps, long every, const double* rho, const double* u0, const double* u_target,
                     double* loss, double* grad_u0, double* grad_force, double grad_omega[6]);
+
+/* The same in device memory of the caller's: `workspace` (256-byte aligned, on
+ * the lattice's device, not in use by work outside the handle's stream) of at
+ * least the `bytes` that lbm_adjoint_workspace returns for these steps, free again
+ * when the call returns.  A program that asks for gradients over and over saves
+ * mapping and unmapping the checkpoints on each call (512^2, 100 states: 1.9 of
+ * 10.8 ms).  workspace == NULL: lbm_adjoint_run.  Errors: as lbm_adjoint_run, and
+ * LBM_EINVAL for a workspace that is too small or misaligned. */
+int lbm_adjoint_workspace(lbm_t h, long nsteps, long every, size_t* bytes);
+int lbm_adjoint_run_in(lbm_t h, long nsteps, long every, const double* rho, const double* u0, const double* u_target,
+                       double* loss, double* grad_u0, double* grad_force, double grad_omega[6], void* workspace,
+                       size_t bytes);
 
 /* ---------------------------------------------------------------------------
  * Batches: many independent lattices advanced together (no counterpart in the

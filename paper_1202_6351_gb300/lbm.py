@@ -75,6 +75,8 @@ SIGNATURES = {
     "lbm_info": (_i, [_vp, C.POINTER(C.c_long), C.POINTER(C.c_size_t), C.POINTER(_vp)]),
     "lbm_bytes_per_update": (C.c_size_t, [_i]),
     "lbm_adjoint_run": (_i, [_vp, _l, _l, _vp, _vp, _vp, _dp, _vp, _vp, _dp]),
+    "lbm_adjoint_workspace": (_i, [_vp, _l, _l, C.POINTER(C.c_size_t)]),
+    "lbm_adjoint_run_in": (_i, [_vp, _l, _l, _vp, _vp, _vp, _dp, _vp, _vp, _dp, _vp, C.c_size_t]),
     "lbm_batch_create": (_i, [C.POINTER(_vp), _i, C.POINTER(_vp)]),
     "lbm_batch_destroy": (_i, [_vp]),
     "lbm_batch_tune": (_i, [_vp, _i, C.POINTER(C.c_float)]),
@@ -359,8 +361,16 @@ class Lattice:
     def info(self):
         return lbm_info(self.h)
 
-    def adjoint_run(self, nsteps, every, u0, u_target, rho=None, want_u0=True, want_force=True):
-        """lbm_adjoint_run with float64 CUDA tensors; returns (loss, grad_u0, grad_force, grad_omega[6])."""
+    def adjoint_workspace(self, nsteps, every) -> int:
+        """Bytes of the device workspace that adjoint_run takes for these steps."""
+        n = C.c_size_t()
+        _check(self.lib.lbm_adjoint_workspace(self.h, int(nsteps), int(every), C.byref(n)))
+        return n.value
+
+    def adjoint_run(self, nsteps, every, u0, u_target, rho=None, want_u0=True, want_force=True, workspace=None):
+        """lbm_adjoint_run with float64 CUDA tensors; returns (loss, grad_u0, grad_force, grad_omega[6]).
+        workspace: a contiguous CUDA tensor of at least adjoint_workspace(nsteps, every) bytes to run in
+        (lbm_adjoint_run_in), or None to allocate it for the call."""
         import torch
 
         shape2 = (2,) + self.shape
@@ -368,10 +378,15 @@ class Lattice:
         gf = torch.empty(shape2, dtype=torch.float64, device="cuda") if want_force else None
         loss = C.c_double()
         gom = (C.c_double * 6)()
-        _check(self.lib.lbm_adjoint_run(
+        ws, nbytes = None, 0
+        if workspace is not None:
+            if not (workspace.is_cuda and workspace.is_contiguous()):
+                raise TypeError("workspace: expected a contiguous CUDA tensor")
+            ws, nbytes = workspace.data_ptr(), workspace.numel() * workspace.element_size()
+        _check(self.lib.lbm_adjoint_run_in(
             self.h, int(nsteps), int(every), _dev(rho, self.shape) if rho is not None else None,
             _dev(u0, shape2), _dev(u_target, shape2), C.byref(loss),
-            gu.data_ptr() if gu is not None else None, gf.data_ptr() if gf is not None else None, gom))
+            gu.data_ptr() if gu is not None else None, gf.data_ptr() if gf is not None else None, gom, ws, nbytes))
         return loss.value, gu, gf, np.array(list(gom))
 
 
