@@ -29,6 +29,32 @@ __device__ __forceinline__ void node_force_any(const Args& a, int force, int x, 
     }
 }
 
+// FP32 <-> FP64 conversions on the integer pipe.  A hardware conversion takes the
+// FP64 pipe (64 cycles per warp and SM quarter), which bounds a kernel that moves 42
+// bytes per node after one or two of them; these take about ten integer instructions
+// for normal numbers and zero and leave the rest to the hardware.  Both give the
+// hardware's result bit for bit (widening is exact; narrowing rounds to nearest even).
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v) {
+    const unsigned b = __float_as_uint(v), e = (b >> 23) & 0xffu;
+    if (e - 1u < 254u) return __hiloint2double(int((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), int(b << 29));
+    if ((b << 1) == 0u) return __hiloint2double(int(b), 0);
+    return double(v);
+}
+template <typename R> __device__ __forceinline__ R narrow_to(double v);
+template <> __device__ __forceinline__ double narrow_to<double>(double v) { return v; }
+template <> __device__ __forceinline__ float narrow_to<float>(double v) {
+    const unsigned hi = unsigned(__double2hiint(v)), lo = unsigned(__double2loint(v));
+    const unsigned e = (hi >> 20) & 0x7ffu, sign = hi & 0x80000000u;
+    if (e - 897u < 253u) {  // a normal FP32 number below the largest binade: rounding up cannot overflow
+        const unsigned keep = ((hi & 0x7fffffffu) - (896u << 20)) << 3 | lo >> 29, rest = lo << 3;
+        const unsigned up = rest > 0x80000000u || (rest == 0x80000000u && (keep & 1u)) ? 1u : 0u;
+        return __uint_as_float(sign | (keep + up));
+    }
+    if (((hi & 0x7fffffffu) | lo) == 0u) return __uint_as_float(sign);
+    return __double2float_rn(v);
+}
+
 // Deviations of node (x, y) at the current time in physical units.
 template <int STORE>
 __device__ __forceinline__ void load_any(const Args& a, bool odd, int x, int y, double d[9]) {
@@ -50,11 +76,24 @@ __device__ __forceinline__ void load_any(const Args& a, bool odd, int x, int y, 
 // w1(+-1) = 1/6 (w = w1(e_x) w1(e_y)):
 //   f_eq - w rho0 = (rho - rho0) w + rho (w1x dphi_y + dphi_x w1y + dphi_x dphi_y).
 // Siblings: the 2nd-order polynomial, f_eq - w rho0 = w (rho - rho0) + w rho (3 eu + 9/2 eu^2 - 3/2 u^2).
+// rho0 in the arithmetic type (the constants hold it times the storage scale, a power of two).
+template <int STORE>
+__device__ __forceinline__ typename Store<STORE>::R rho0_of(const Args& a) {
+    if constexpr (STORE == LBM_F64) return a.rho0;
+    else return a.kf[K_RHO0] * float(1.0 / Store<STORE>::scale);
+}
+
 template <typename R>
 __device__ __forceinline__ R w1(int e) { return e == 0 ? R(2.0 / 3.0) : R(1.0 / 6.0); }
 template <typename R>
 __device__ __forceinline__ R dphi(int e, R u) { return e == 0 ? -u * u : R(0.5) * (u * u + R(e) * u); }
 
+//
+// Bound by HBM (24 bytes read and 9 stored elements per node) once the FP64 pipe is
+// out of the way: rho0 and a uniform force come converted, the fields are narrowed on
+// the integer pipe, and the source terms are formed only under a force (8192^2, us
+// before -> now: FP32 803 -> 730, FP16 803 -> 676; macros_kernel, where conversions and
+// a zero force took all eight FP64 instructions: FP32 1100 -> 566, FP16 1097 -> 489).
 template <int STORE>
 __global__ void init_kernel(const Args a, int model, int force, bool ffield_double, const double* rho,
                             const double* u) {
@@ -64,13 +103,15 @@ __global__ void init_kernel(const Args a, int model, int force, bool ffield_doub
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
     if (x >= a.nx) return;
     const long long n = (long long)y * a.nx + x, p = (long long)a.nx * a.ny;
-    const R dr = R(rho ? rho[n] - a.rho0 : 0.0);
-    const R r = R(a.rho0) + dr;
-    const R ux = R(u ? u[n] : 0.0), uy = R(u ? u[p + n] : 0.0);
-    double Fxd, Fyd;
-    node_force_any(a, force, x, y, Fxd, Fyd, ffield_double);
-    R Sq[9];
-    source<R>(ux, uy, R(Fxd), R(Fyd), Sq);
+    const R dr = rho ? narrow_to<R>(rho[n] - a.rho0) : R(0);
+    const R r = rho0_of<STORE>(a) + dr;
+    const R ux = u ? narrow_to<R>(u[n]) : R(0), uy = u ? narrow_to<R>(u[p + n]) : R(0);
+    R Sq[9] = {R(0), R(0), R(0), R(0), R(0), R(0), R(0), R(0), R(0)};
+    if (force != 0) {
+        double Fx, Fy;
+        node_force_any(a, force, x, y, Fx, Fy, ffield_double);
+        source<R>(ux, uy, R(Fx), R(Fy), Sq);
+    }
     T* f = static_cast<T*>(a.f);
     const long long off = (long long)y * a.pitch + x;
     const R usq = R(1.5) * (ux * ux + uy * uy);
@@ -134,14 +175,20 @@ __device__ __forceinline__ void node_rho_u(const Args& a, bool odd, int force, b
 #pragma unroll
         for (int q = 0; q < 9; ++q) d[q] *= R(1.0 / Store<STORE>::scale);
     }
-    const Moments<R> m = moments<R>(d, R(a.rho0));
-    double Fx, Fy;
-    node_force_any(a, force, x, y, Fx, Fy, ffd);
-    const R px = m.jx + R(0.5 * Fx), py = m.jy + R(0.5 * Fy);
-    const R rr = R(a.rho0) + m.drho;
-    rho = a.rho0 + double(m.drho);
-    ux = double(px / rr);
-    uy = double(py / rr);
+    const R rho0 = rho0_of<STORE>(a);
+    const Moments<R> m = moments<R>(d, rho0);
+    R hx = R(0), hy = R(0);
+    if (force != 0) {
+        double Fx, Fy;
+        node_force_any(a, force, x, y, Fx, Fy, ffd);
+        hx = R(0.5 * Fx);
+        hy = R(0.5 * Fy);
+    }
+    const R px = m.jx + hx, py = m.jy + hy;
+    const R rr = rho0 + m.drho;
+    rho = a.rho0 + widen(m.drho);
+    ux = widen(px / rr);
+    uy = widen(py / rr);
 }
 
 template <int STORE>
