@@ -15,10 +15,9 @@
 // (the template arguments of the tile body).  The tile list is ordered by
 // class and each class has a kernel of its own, so every kernel carries one
 // tile body under its register budget, as the single-lattice kernel does; the
-// kernels of one two-step launch are independent and run side by side.  Every
-// class collides one node per thread: the packed FP32x2 node pairs of the
-// single-lattice kernel spill here (the tile decode takes registers of its
-// own) and ran slower.
+// kernels of one launch are independent and run side by side.  A batch whose
+// lattices all take the unforced cascaded collision with round to nearest runs
+// the multi-step tile instead (batch_multi_kernel).
 #pragma once
 
 #include <utility>
@@ -79,7 +78,7 @@ __global__ void __launch_bounds__(FusedTile<STORE>::THREADS, FusedTile<STORE>::M
     const unsigned rb0 = SR ? rtab[dom * rstride + 2 * kstep] : 0u;
     const unsigned rb1 = SR ? rtab[dom * rstride + 2 * kstep + 1] : 0u;
     const int src = k & 1;
-    fused2_tile<MODEL, STORE, FORCE, WALLS, SR, false>(&P.map[src], sdom.a, P.arr[src], P.arr[src ^ 1], err,
+    fused2_tile<MODEL, STORE, FORCE, WALLS, SR>(&P.map[src], sdom.a, P.arr[src], P.arr[src ^ 1], err,
                                                        tx * kBatchFusedTX, ty * kBatchFusedTY, rb0, rb1, fused_smem,
                                                        &bar, &ok);
 }
