@@ -303,16 +303,17 @@ bool same_launch(const Args& x, const Args& y) {
 cudaError_t launch_resident(const lbm_s* h, int n) {
     const unsigned long long t = static_cast<unsigned long long>(h->t);
     switch (h->store) {
+        case LBM_F64: return lbm::launch_resident_f64(h->a, h->model, force_mode(h), t, n, h->stream);
         case LBM_F32: return lbm::launch_resident_f32(h->a, h->model, force_mode(h), t, n, h->stream);
         case LBM_BF16DEV: return lbm::launch_resident_bf16(h->a, h->model, force_mode(h), t, n, h->stream);
         default: return lbm::launch_resident_f16(h->a, h->model, force_mode(h), t, n, h->stream);
     }
 }
 
-// Small FP32 and 16-bit lattices step on chip, whatever the variant (the results are
+// Small lattices step on chip, whatever the variant (the results are
 // those of variants 0, 2 and 3); variant 1, which rounds differently, stays itself.
 bool resident_active(lbm_s* h) {
-    if (h->store == LBM_F64 || h->a.variant == 1 || !lbm::resident_fits(h->a)) return false;
+    if (h->a.variant == 1 || !lbm::resident_fits(h->a, h->store)) return false;
     if (h->resident < 0) {
         h->resident = launch_resident(h, 0) == cudaSuccess ? 1 : 0;
         if (!h->resident) cudaGetLastError();

@@ -72,6 +72,7 @@ cudaError_t launch_multi_f16(const CUtensorMap& map, const Args& a, void* out, i
 
 // Steps t0 .. t0 + n - 1 of a small lattice in one launch (lbm_resident.cuh); n = 0
 // only asks whether the device can run it.
+cudaError_t launch_resident_f64(const Args& a, int model, int force, unsigned long long t0, int n, cudaStream_t s);
 cudaError_t launch_resident_f32(const Args& a, int model, int force, unsigned long long t0, int n, cudaStream_t s);
 cudaError_t launch_resident_bf16(const Args& a, int model, int force, unsigned long long t0, int n, cudaStream_t s);
 cudaError_t launch_resident_f16(const Args& a, int model, int force, unsigned long long t0, int n, cudaStream_t s);

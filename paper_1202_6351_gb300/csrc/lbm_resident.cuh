@@ -1,5 +1,5 @@
 // lbm_resident.cuh -- many time steps per launch for a small lattice that stays on
-// chip (FP32 and 16-bit storage, every collision, force, edge and rounding).
+// chip (every storage kind, collision, force, edge and rounding).
 //
 // Up to about 100^2 nodes a step takes less than the gap between two launches (FP32
 // 64^2: 1.3 us per step from a graph, of which the update is 0.3).  Here one cluster
@@ -15,11 +15,15 @@
 // instruction issue of five warps per SM quarter at most, so the lattice is spread
 // over as many CTAs as a cluster takes (64^2 cavity: 0.87 us with 8, 0.69 with 16).
 // Beyond one node per thread (800 a CTA, 80 registers each) a launch per step over
-// all 152 SMs wins: 128^2 1.8 us here with two rounds, 1.5 there.  FP64 gains nothing
-// (the FP64 pipe of 16 SMs instead of all).
+// all 152 SMs wins: 128^2 1.8 us here with two rounds, 1.5 there.  An FP64 step costs its
+// instructions (64 cycles each per warp and SM quarter), so beyond 128 nodes a CTA,
+// one warp per quarter, the launch over all SMs wins; up to there what is saved is
+// the launch and the filling of the chip.
 // us per step, before -> now: FP32 periodic 16^2 1.2 -> 0.43, 64^2 1.3 -> 0.52, 101^2
 // 1.35 -> 0.86; cavity 26^2 1.5 -> 0.64, 64^2 1.5 -> 0.69, 101^2 1.55 -> 1.02; raw-MRT forced
-// cavity 101^2 1.6 -> 1.15.
+// cavity 101^2 1.6 -> 1.15; FP64 forced channel 4 x 32 5.87 -> 5.18, periodic 32^2 4.49 ->
+// 3.77, cavity 32^2 5.35 -> 4.38, 128 x 16 5.22 -> 4.87 (128 nodes a CTA); in calls of 8 steps
+// 4 x 32 5.96 -> 5.43, 128 x 16 5.37 -> 5.12.
 #pragma once
 
 #include "lbm_async.cuh"
@@ -27,9 +31,11 @@
 
 namespace lbm {
 
-constexpr int kResidentThreads = 800;     // most threads of a CTA: 80 registers each
+// Most threads of a CTA: 80 registers each; FP64 one warp per SM quarter (every further
+// warp there costs as much as the first).
+constexpr int resident_threads(int store) { return store == LBM_F64 ? 128 : 800; }
 constexpr int kResidentMinSteps = 8;      // below, filling and emptying shared memory costs more than it saves
-constexpr long kResidentMaxSteps = 16384; // of one launch (about 10 ms)
+constexpr long kResidentMaxSteps = 16384; // of one launch (about 10 ms, FP64 100)
 
 // CTAs of the cluster: a power of two, at most one per row.
 inline int resident_size(const Args& a) {
@@ -37,9 +43,9 @@ inline int resident_size(const Args& a) {
     while (size > a.ny) size /= 2;
     return size;
 }
-inline bool resident_fits(const Args& a) {
+inline bool resident_fits(const Args& a, int store) {
     const int size = resident_size(a);
-    return (long long)((a.ny + size - 1) / size) * a.nx <= kResidentThreads;
+    return (long long)((a.ny + size - 1) / size) * a.nx <= resident_threads(store);
 }
 
 __device__ __forceinline__ unsigned cluster_rank() {
@@ -65,7 +71,11 @@ __device__ __forceinline__ void cluster_sync() {
 // shared memory by its plain address.
 template <typename T> __device__ __forceinline__ T own_load(unsigned addr) {
     T v;
-    if constexpr (sizeof(T) == 4) {
+    if constexpr (sizeof(T) == 8) {
+        unsigned long long w;
+        asm volatile("ld.shared.b64 %0, [%1];" : "=l"(w) : "r"(addr) : "memory");
+        __builtin_memcpy(&v, &w, 8);
+    } else if constexpr (sizeof(T) == 4) {
         unsigned w;
         asm volatile("ld.shared.b32 %0, [%1];" : "=r"(w) : "r"(addr) : "memory");
         __builtin_memcpy(&v, &w, 4);
@@ -77,7 +87,11 @@ template <typename T> __device__ __forceinline__ T own_load(unsigned addr) {
     return v;
 }
 template <typename T> __device__ __forceinline__ void own_store(unsigned addr, T v) {
-    if constexpr (sizeof(T) == 4) {
+    if constexpr (sizeof(T) == 8) {
+        unsigned long long w;
+        __builtin_memcpy(&w, &v, 8);
+        asm volatile("st.shared.b64 [%0], %1;" ::"r"(addr), "l"(w) : "memory");
+    } else if constexpr (sizeof(T) == 4) {
         unsigned w;
         __builtin_memcpy(&w, &v, 4);
         asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(w) : "memory");
@@ -89,7 +103,11 @@ template <typename T> __device__ __forceinline__ void own_store(unsigned addr, T
 }
 template <typename T> __device__ __forceinline__ T cluster_load(unsigned addr) {
     T v;
-    if constexpr (sizeof(T) == 4) {
+    if constexpr (sizeof(T) == 8) {
+        unsigned long long w;
+        asm volatile("ld.shared::cluster.b64 %0, [%1];" : "=l"(w) : "r"(addr) : "memory");
+        __builtin_memcpy(&v, &w, 8);
+    } else if constexpr (sizeof(T) == 4) {
         unsigned w;
         asm volatile("ld.shared::cluster.b32 %0, [%1];" : "=r"(w) : "r"(addr) : "memory");
         __builtin_memcpy(&v, &w, 4);
@@ -101,7 +119,11 @@ template <typename T> __device__ __forceinline__ T cluster_load(unsigned addr) {
     return v;
 }
 template <typename T> __device__ __forceinline__ void cluster_store(unsigned addr, T v) {
-    if constexpr (sizeof(T) == 4) {
+    if constexpr (sizeof(T) == 8) {
+        unsigned long long w;
+        __builtin_memcpy(&w, &v, 8);
+        asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(addr), "l"(w) : "memory");
+    } else if constexpr (sizeof(T) == 4) {
         unsigned w;
         __builtin_memcpy(&w, &v, 4);
         asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(w) : "memory");
@@ -171,7 +193,7 @@ __device__ __forceinline__ void resident_node(const Args& a, const Coef<typename
 // Steps t0 .. t0 + n - 1 of the whole lattice in place.  One cluster; CTA k holds
 // ny / size rows (+ 1 for the first ny mod size CTAs), one thread per node.
 template <int MODEL, int STORE, int FORCE, bool SR>
-__global__ void __launch_bounds__(kResidentThreads, 1) resident_kernel(const Args a, unsigned long long t0, int n, int rows_max) {
+__global__ void __launch_bounds__(resident_threads(STORE), 1) resident_kernel(const Args a, unsigned long long t0, int n, int rows_max) {
     using T = typename Store<STORE>::T;
     using R = typename Store<STORE>::R;
     extern __shared__ __align__(16) unsigned char resident_smem[];
@@ -259,8 +281,10 @@ static cudaError_t launch_resident_one(const Args& a, unsigned long long t0, int
 
 template <int MODEL, int STORE, int FORCE>
 static cudaError_t launch_resident_sr(const Args& a, unsigned long long t0, int n, cudaStream_t s) {
-    return a.rseed ? launch_resident_one<MODEL, STORE, FORCE, true>(a, t0, n, s)
-                   : launch_resident_one<MODEL, STORE, FORCE, false>(a, t0, n, s);
+    if constexpr (STORE != LBM_F64) {
+        if (a.rseed) return launch_resident_one<MODEL, STORE, FORCE, true>(a, t0, n, s);
+    }
+    return launch_resident_one<MODEL, STORE, FORCE, false>(a, t0, n, s);
 }
 template <int MODEL, int STORE>
 static cudaError_t launch_resident_force(const Args& a, int force, unsigned long long t0, int n, cudaStream_t s) {

@@ -93,3 +93,19 @@ def test_divergence_checks_fall_on_the_same_steps():
                     L.step(n)
             assert err.value.code == lbm.LBM_EDIVERGED
             assert L.time % 20 == 0
+
+
+# FP64: 128 nodes per CTA
+F64_SHAPES = [(1, 1), (5, 1), (128, 1), (129, 1), (1, 40), (2, 2), (4, 4), (4, 32), (37, 5), (33, 15), (31, 17), (16, 128), (64, 32),
+              (42, 48), (128, 16), (129, 16), (3, 600)]
+
+
+@pytest.mark.parametrize("force", ["none", "uniform", "field"])
+@pytest.mark.parametrize("model", [lbm.CASCADED, lbm.BGK, lbm.RAWMRT], ids=["cascaded", "bgk", "rawmrt"])
+@pytest.mark.parametrize("shape", F64_SHAPES, ids=[f"{a}x{b}" for a, b in F64_SHAPES])
+def test_on_chip_f64_steps_are_bitwise_equal_to_single_launches(shape, model, force):
+    for edges in EDGES:
+        whole = run(shape, edges, model, lbm.F64, force, False, (9, 16))
+        single = run(shape, edges, model, lbm.F64, force, False, (1,) * 25)
+        for a, b in zip(whole, (single[8], single[24])):
+            np.testing.assert_array_equal(a, b)
