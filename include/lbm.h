@@ -194,7 +194,8 @@ int lbm_init_device(lbm_t h, const double* rho, const double* u);
  * of at least lbm_set_graph_steps steps starting at an even step are replayed
  * from a CUDA graph on an internal stream that is ordered after the handle's
  * stream and before any later work on it (the graph is recaptured whenever a
- * rate, force, force field, variant or rounding mode has changed).  With the divergence
+ * rate, force, force field, variant or rounding mode has changed, and under
+ * variant 3 when the divergence check was switched on or off).  With the divergence
  * check on (lbm_set_check) the call synchronises at every
  * check and returns LBM_EDIVERGED when it fails. */
 int lbm_step(lbm_t h, long n);

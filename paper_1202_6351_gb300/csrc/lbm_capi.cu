@@ -326,7 +326,7 @@ void drop_graph(lbm_s* h) {
     h->graph = nullptr;
 }
 
-// Captures graph_steps launches (even parity first) on the internal stream.
+// Captures graph_len(h) steps (even parity first) on the internal stream.
 cudaError_t capture_graph(lbm_s* h, int fm) {
     drop_graph(h);
     cudaError_t e = cudaSuccess;
@@ -376,16 +376,20 @@ cudaError_t capture_graph(lbm_s* h, int fm) {
     if (e == cudaSuccess) {
         h->graph_args = h->a;
         h->graph_force = fm;
+        h->graph_replay = len;
+        h->graph_fused = fused;
     }
     return e;
 }
 
-// graph_steps steps from an even step: ordered after prior work on h->stream,
+// graph_len(h) steps from an even step: ordered after prior work on h->stream,
 // and later work on h->stream waits for them.
 cudaError_t replay_graph(lbm_s* h) {
     const int fm = force_mode(h);
     cudaError_t e = cudaSuccess;
-    if (!h->graph || fm != h->graph_force || !same_launch(h->a, h->graph_args)) e = capture_graph(h, fm);
+    if (!h->graph || fm != h->graph_force || graph_len(h) != h->graph_replay || fused_active(h) != h->graph_fused ||
+        !same_launch(h->a, h->graph_args))
+        e = capture_graph(h, fm);
     if (e == cudaSuccess) e = cudaEventRecord(h->ev_in, h->stream);
     if (e == cudaSuccess) e = cudaStreamWaitEvent(h->gstream, h->ev_in, 0);
     if (e == cudaSuccess && h->a.rseed) {

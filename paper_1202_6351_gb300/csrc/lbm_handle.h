@@ -24,13 +24,16 @@ struct lbm_s {
     double check_rtol = 0.0, mass0 = 0.0;
     // CUDA-graph replay of lbm_step: `graph_steps` launches captured from an even
     // step on an internal stream, ordered against `stream` by two events; the
-    // launch arguments it was captured with are kept to detect any change.
+    // launch arguments, the steps of a replay and the kind of launch it was captured
+    // with (two-step launches, or single steps while the divergence check is on) are
+    // kept to detect any change.
     int graph_steps = 64;
     cudaGraphExec_t graph = nullptr;
     cudaStream_t gstream = nullptr;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
     lbm::Args graph_args{};
-    int graph_force = -1;
+    int graph_force = -1, graph_replay = 0;
+    bool graph_fused = false;
     // Stochastic rounding of 16-bit stores (lbm_set_rounding): per-step hashes
     // C0 of a graph replay, filled on the graph stream before each replay.
     unsigned* d_rtable = nullptr;
