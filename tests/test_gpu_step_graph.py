@@ -63,3 +63,33 @@ def test_switching_the_check_recaptures_the_step_graph(kind, graph_steps, checks
     for (ta, fa), (tb, fb) in zip(whole, single):
         assert ta == tb
         np.testing.assert_array_equal(fa, fb)
+
+
+@pytest.mark.parametrize("edges,force", [("periodic", (0.0, 0.0)), ("cavity", (0.0, 0.0)), ("cavity", (2e-5, 1e-5))])
+@pytest.mark.parametrize("stochastic", [False, True], ids=["nearest", "stochastic"])
+@pytest.mark.parametrize("store", [lbm.F32, lbm.F16DEV, lbm.BF16DEV, lbm.F64], ids=["f32", "f16", "bf16", "f64"])
+@pytest.mark.parametrize("shape", [(257, 70), (403, 45)], ids=["257x70", "403x45"])
+def test_replays_are_bitwise_equal_to_single_launches(shape, store, stochastic, edges, force):
+    """Every variant that rounds alike, at two replay lengths, from odd and even steps and
+    across a change of rates."""
+    if stochastic and store == lbm.F64:
+        pytest.skip("FP64 storage rounds to nearest only")
+
+    def run(variant, graph, split):
+        with lattice(*shape, store, edges=edges, force=force, stochastic=stochastic) as L:
+            L.set_variant(variant).set_graph_steps(graph)
+            out = []
+            for n in (3, 37, 66):
+                for k in ([1] * n if split else [n]):
+                    L.step(k)
+                out.append(L.get_f())
+                L.set_omegas((1.0, 1.5, 1.5, 1.0, 1.1, 1.0))
+            assert L.time == 106
+            return out
+
+    ref = run(0, 0, True)
+    variants = {lbm.F64: (0,), lbm.F32: (0, 3)}.get(store, (0, 2, 3))
+    for variant in variants:
+        for graph in (8, 64):
+            for k, (a, b) in enumerate(zip(run(variant, graph, False), ref)):
+                np.testing.assert_array_equal(a, b, err_msg=f"variant {variant}, graph {graph}, chunk {k}")
