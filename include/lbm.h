@@ -280,7 +280,8 @@ int lbm_adjoint_run(lbm_t h, long nsteps, long every, const double* rho, const d
  * when the call returns.  A program that asks for gradients over and over saves
  * mapping and unmapping the checkpoints on each call (512^2, 100 states: 1.9 of
  * 10.8 ms).  workspace == NULL: lbm_adjoint_run.  Errors: as lbm_adjoint_run, and
- * LBM_EINVAL for a workspace that is too small or misaligned. */
+ * LBM_EINVAL for a workspace that is too small or misaligned; LBM_ENOMEM from
+ * either call if the bytes exceed the range of their type. */
 int lbm_adjoint_workspace(lbm_t h, long nsteps, long every, size_t* bytes);
 int lbm_adjoint_run_in(lbm_t h, long nsteps, long every, const double* rho, const double* u0, const double* u_target,
                        double* loss, double* grad_u0, double* grad_force, double grad_omega[6], void* workspace,

@@ -263,7 +263,7 @@ cudaError_t run_reverse(lbm_s* h, long nsteps, long every, const double* rho, co
     const int fm = force_mode(h);
     const size_t SB = h->state_bytes;
     const dim3 grid((a.nx + kThreads - 1) / kThreads, a.ny);
-    const long nck = (nsteps + every - 1) / every;
+    const long nck = (nsteps - 1) / every + 1;
     cudaError_t e;
 
     // Forward pass.  f^t lives in ckpt[c] at the checkpoint times t = c every and
@@ -337,12 +337,16 @@ namespace {
 // What a run keeps on the device besides its results: checkpoints, recomputed states of a
 // segment, two adjoint arrays, partial sums of rates and loss, the force gradient (if
 // the caller takes none) and its FP32 segment sum.  Offsets are multiples of 256 bytes.
+// `fits` is false if the sum leaves the range of a byte count (at most a quarter of it,
+// so that no partial sum wraps around).
 struct AdjointSpace {
     size_t ckpt, seg, lam0, lam1, acc, gc, lossp, gF, gseg, total;
-    AdjointSpace(const lbm_s* h, long nsteps, long every) {
+    bool fits;
+    AdjointSpace(const lbm_s* h, long nsteps, long every) {  // every <= nsteps
         const size_t SB = h->state_bytes, n = (size_t)h->a.nx * h->a.ny;
-        const size_t nck = size_t((nsteps + every - 1) / every), seglen = size_t(std::min(every, nsteps));
+        const size_t nck = size_t((nsteps - 1) / every + 1), nseg = std::max(size_t(1), size_t(every) - 1);
         const bool dbl = h->store == LBM_F64;
+        fits = nck + nseg <= SIZE_MAX / 4 / SB;  // the rest is below 2^41 bytes
         total = 0;
         auto take = [&](size_t bytes) {
             const size_t at = total;
@@ -350,7 +354,7 @@ struct AdjointSpace {
             return at;
         };
         ckpt = take(nck * SB);
-        seg = take(std::max(size_t(1), seglen - 1) * SB);
+        seg = take(nseg * SB);
         const size_t lam = 9 * (size_t)h->a.plane * (dbl ? 8 : 4);
         lam0 = take(lam);
         lam1 = take(lam);
@@ -373,12 +377,18 @@ int adjoint_admitted(lbm_t h, long nsteps, long every) {
     return LBM_OK;
 }
 
+int too_many_states(long nsteps, long every) {
+    return lbm::set_error(LBM_ENOMEM, "lbm_adjoint_run: the states of %ld steps, one checkpoint per %ld, exceed any memory", nsteps, every);
+}
+
 }  // namespace
 
 extern "C" int lbm_adjoint_workspace(lbm_t h, long nsteps, long every, size_t* bytes) {
     if (const int rc = adjoint_admitted(h, nsteps, every)) return rc;
     if (!bytes) return lbm::set_error(LBM_EINVAL, "lbm_adjoint_workspace: bytes is NULL");
-    *bytes = AdjointSpace(h, nsteps, every).total;
+    const AdjointSpace at(h, nsteps, std::min(every, nsteps));
+    if (!at.fits) return too_many_states(nsteps, every);
+    *bytes = at.total;
     return LBM_OK;
 }
 
@@ -394,7 +404,9 @@ extern "C" int lbm_adjoint_run_in(lbm_t h, long nsteps, long every, const double
     using namespace lbm;
     if (const int rc = adjoint_admitted(h, nsteps, every)) return rc;
     if (!u0 || !u_target || !loss) return set_error(LBM_EINVAL, "lbm_adjoint_run: u0, u_target and loss are required");
+    every = std::min(every, nsteps);  // a longer interval is one segment
     const AdjointSpace at(h, nsteps, every);
+    if (!at.fits) return too_many_states(nsteps, every);
     if (workspace && (bytes < at.total || reinterpret_cast<uintptr_t>(workspace) % 256 != 0))
         return set_error(LBM_EINVAL, "lbm_adjoint_run_in: the workspace needs %zu bytes at a 256-byte boundary", at.total);
     int prev = -1;
