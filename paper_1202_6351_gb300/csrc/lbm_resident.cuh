@@ -253,9 +253,11 @@ template <int MODEL, int STORE, int FORCE, bool SR>
 static cudaError_t launch_resident_one(const Args& a, unsigned long long t0, int n, cudaStream_t s) {
     const int size = resident_size(a), rows_max = (a.ny + size - 1) / size;
     const size_t smem = size_t(9) * rows_max * a.nx * sizeof(typename Store<STORE>::T);
+    // At most 28,800 bytes a CTA, so no shared memory has to be opted into.  A function's
+    // attributes belong to all lattices and host threads: only ever set to one value.
+    static_assert(size_t(9) * resident_threads(STORE) * sizeof(typename Store<STORE>::T) <= 48 * 1024, "no opt-in");
     auto kernel = resident_kernel<MODEL, STORE, FORCE, SR>;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    if (e == cudaSuccess && size > 8) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
