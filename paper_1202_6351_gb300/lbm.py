@@ -223,9 +223,9 @@ class Lattice:
 
     # lifetime
     def close(self):
-        if self.h is not None:
-            lbm_destroy(self.h)
-            self.h = None
+        h, self.h = self.h, None  # freed by the call also where it reports an error
+        if h is not None:
+            lbm_destroy(h)
 
     def __del__(self):
         try:
@@ -407,9 +407,9 @@ class Batch:
         _check(self.lib.lbm_batch_create(arr, len(self.lattices), C.byref(self.b)))
 
     def close(self):
-        if self.b is not None:
-            _check(self.lib.lbm_batch_destroy(self.b))
-            self.b = None
+        b, self.b = self.b, None
+        if b is not None:
+            _check(self.lib.lbm_batch_destroy(b))
 
     def __del__(self):
         try:
@@ -470,9 +470,9 @@ class Lattice3:
             _check(self.lib.lbm3_set_stream(self.h, C.c_void_p(stream)))
 
     def close(self):
-        if self.h is not None:
-            _check(self.lib.lbm3_destroy(self.h))
-            self.h = None
+        h, self.h = self.h, None
+        if h is not None:
+            _check(self.lib.lbm3_destroy(h))
 
     def __del__(self):
         try:
