@@ -118,9 +118,9 @@ inline bool adj_serial_rows(const Args& a) { return (long long)a.nx * a.ny >= (1
 
 template <int ST, int RPT>
 __global__ void __launch_bounds__(kThreads, ST == LBM_F32 ? 7 : 1) adj_step_kernel(const Args a, bool odd, int force,
-                                                            const typename Store<ST>::R* __restrict__ lin,
-                                                            typename Store<ST>::R* __restrict__ lout,
-                                                            typename Store<ST>::R* __restrict__ gs, bool first,
+                                                            const typename Store<ST>::R* lin,
+                                                            typename Store<ST>::R* lout,
+                                                            typename Store<ST>::R* gs, bool first,
                                                             double* gc) {
     using R = typename Store<ST>::R;
     constexpr int COLS = adj_cols(RPT);

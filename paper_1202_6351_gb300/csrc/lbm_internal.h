@@ -14,7 +14,8 @@ namespace lbm {
 // kernel before: the next grid is set up while the last blocks finish, and
 // every kernel launched this way calls pdl_wait, which returns when the grid
 // before has completed and its writes are visible, before it touches global
-// memory.  No kernel asks for the next one earlier (launch_dependents): blocks
+// memory.  Its pointer arguments are not __restrict__: the memory is written by
+// others while it waits.  No kernel asks for the next one earlier (launch_dependents): blocks
 // placed while the current grid still holds most slots end up unevenly spread
 // over the SMs (FP32 257^2: 2.35 us per step so, 1.92 without; 2.16 without any
 // overlap).

@@ -353,8 +353,7 @@ __device__ __forceinline__ void multi_tile(const CUtensorMap* map, const Args& a
 
 template <class G>
 __global__ void __launch_bounds__(G::NT, G::MINB)
-    multi_kernel(const __grid_constant__ CUtensorMap map, const Args a, const void* __restrict__ in, void* __restrict__ out,
-                 int* __restrict__ err, int steps) {
+    multi_kernel(const __grid_constant__ CUtensorMap map, const Args a, const void* in, void* out, int* err, int steps) {
     extern __shared__ __align__(1024) unsigned char multi_smem[];
     __shared__ __align__(8) unsigned long long bar;
     __shared__ int ok;
