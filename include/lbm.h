@@ -161,7 +161,9 @@ int lbm_set_rounding(lbm_t h, int mode, unsigned long long seed);
  * variant 3 has fixed tiles) on the lattice itself (the state is snapshot
  * and restored, so it is left unchanged) and keeps the fastest pair; ms (may
  * be NULL) receives the best time per step of variants 0..3 (0 where not run).
- * Synchronous. */
+ * A lattice that lbm_step steps on chip is timed that way (at least 8 steps);
+ * variants 0, 2 and 3 are then one kernel and share its time, and variant 0
+ * stands for them.  Synchronous. */
 #define LBM_NUM_VARIANTS 4
 int lbm_tune(lbm_t h, int trial_steps, float ms[LBM_NUM_VARIANTS]);
 

@@ -299,9 +299,9 @@ bool same_launch(const Args& x, const Args& y) {
     return true;
 }
 
-// Steps h->t .. h->t + n - 1 by the small-lattice kernel.
-cudaError_t launch_resident(const lbm_s* h, int n) {
-    const unsigned long long t = static_cast<unsigned long long>(h->t);
+// Steps t0 .. t0 + n - 1 by the small-lattice kernel (n = 0: can the device run it?).
+cudaError_t launch_resident(const lbm_s* h, long t0, int n) {
+    const unsigned long long t = static_cast<unsigned long long>(t0);
     switch (h->store) {
         case LBM_F64: return lbm::launch_resident_f64(h->a, h->model, force_mode(h), t, n, h->stream);
         case LBM_F32: return lbm::launch_resident_f32(h->a, h->model, force_mode(h), t, n, h->stream);
@@ -315,7 +315,7 @@ cudaError_t launch_resident(const lbm_s* h, int n) {
 bool resident_active(lbm_s* h) {
     if (h->a.variant == 1 || !lbm::resident_fits(h->a, h->store)) return false;
     if (h->resident < 0) {
-        h->resident = launch_resident(h, 0) == cudaSuccess ? 1 : 0;
+        h->resident = launch_resident(h, h->t, 0) == cudaSuccess ? 1 : 0;
         if (!h->resident) cudaGetLastError();
     }
     return h->resident == 1;
@@ -623,18 +623,22 @@ int lbm_tune(lbm_t h, int trial_steps, float ms[LBM_NUM_VARIANTS]) {
         for (int v = 0; v < LBM_NUM_VARIANTS; ++v) ms[v] = 0.f;
     static const int widths[3] = {128, 64, 32};  // CTA shapes 128x1, 64x2, 32x4
     const int v_prev = h->a.variant;
-    // `steps` steps from step h->t as lbm_step takes them without graphs
-    auto run = [&](int k0, int count) -> cudaError_t {
+    // `count` steps from step h->t + k0 as lbm_step takes them without graphs; where it steps on chip,
+    // as a call long enough for that
+    auto run = [&](long k0, long count) -> cudaError_t {
         cudaError_t e = cudaSuccess;
+        const bool resident = resident_active(h);
         for (long t = h->t + k0, end = h->t + k0 + count; t < end && e == cudaSuccess;) {
-            if (fused_active(h) && (t & 1) == 0 && end - t >= 2) {
-                int took = 0;
+            int took = 1;
+            if (resident) {
+                took = int(std::min(end - t, lbm::kResidentMaxSteps));
+                e = launch_resident(h, t, took);
+            } else if (fused_active(h) && (t & 1) == 0 && end - t >= 2) {
                 e = launch_fused_at(h, t, end - t, &took);
-                t += took;
             } else {
                 e = launch_step_at(h, (t & 1) != 0, t);
-                t += 1;
             }
+            t += took;
         }
         return e;
     };
@@ -646,30 +650,41 @@ int lbm_tune(lbm_t h, int trial_steps, float ms[LBM_NUM_VARIANTS]) {
     if (e == cudaSuccess) e = cudaEventCreate(&t1);
     float best = 1e30f;
     int best_v = 0, best_w = 128;
+    h->a.variant = 0;
+    const bool chip = resident_active(h);  // then variants 0, 2 and 3 are one kernel, timed as variant 0
+    float chip_ms = 0.f;
     for (int v = 0; v < LBM_NUM_VARIANTS && e == cudaSuccess; ++v) {
         if (!variant_allowed(h->store, v)) continue;
+        if (chip && v >= 2) {
+            if (ms && (v == 2 || h->check_every == 0)) ms[v] = chip_ms;
+            continue;
+        }
         if (v == 3 && (ensure_fused(h) != cudaSuccess || h->check_every != 0)) {
             cudaGetLastError();  // no room for the second array: variant 3 is not a candidate
             continue;
         }
         float best_of_v = 1e30f;
-        for (int wi = 0; wi < (v == 3 ? 1 : 3) && e == cudaSuccess; ++wi) {  // variant 3 has a fixed tile
+        const bool fixed = v == 3 || (chip && v == 0);  // one shape
+        const int count = chip && v == 0 ? std::max(steps, lbm::kResidentMinSteps) : steps;
+        for (int wi = 0; wi < (fixed ? 1 : 3) && e == cudaSuccess; ++wi) {
             h->a.variant = v;
             h->a.block_x = widths[wi];
             e = run(0, 2);
             if (e == cudaSuccess) e = cudaEventRecord(t0, h->stream);
-            if (e == cudaSuccess) e = run(2, steps);
+            if (e == cudaSuccess) e = run(2, count);
             if (e == cudaSuccess) e = cudaEventRecord(t1, h->stream);
             if (e == cudaSuccess) e = cudaEventSynchronize(t1);
             float t = 0.f;
             if (e == cudaSuccess) e = cudaEventElapsedTime(&t, t0, t1);
             if (e == cudaSuccess) {
-                best_of_v = std::min(best_of_v, t / steps);
+                t /= count;
+                best_of_v = std::min(best_of_v, t);
                 if (t < best) { best = t; best_v = v; best_w = widths[wi]; }
                 e = cudaMemcpyAsync(h->state, backup, h->state_bytes, cudaMemcpyDeviceToDevice, h->stream);
             }
         }
         if (ms && e == cudaSuccess) ms[v] = best_of_v;
+        if (chip && v == 0) chip_ms = best_of_v;
     }
     h->a.variant = e == cudaSuccess ? best_v : v_prev;
     h->a.block_x = best_w;
@@ -776,7 +791,7 @@ int lbm_step(lbm_t h, long n) {
         int took = 1;
         if (resident && left >= lbm::kResidentMinSteps) {
             took = int(std::min(left, lbm::kResidentMaxSteps));
-            LBM_CUDA(launch_resident(h, took), "small-lattice steps");
+            LBM_CUDA(launch_resident(h, h->t, took), "small-lattice steps");
         } else if (len > 0 && (h->t & 1) == 0 && left >= len) {
             took = len;
             LBM_CUDA(replay_graph(h), "step graph");
