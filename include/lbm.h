@@ -157,8 +157,8 @@ int lbm_set_variant(lbm_t h, int variant);
 int lbm_set_rounding(lbm_t h, int mode, unsigned long long seed);
 
 /* Autotuner for one lattice: times `trial_steps` steps of each kernel variant
- * the storage admits with each CTA shape (128x1, 64x2, 32x4 threads;
- * variant 3 has fixed tiles) on the lattice itself (the state is snapshot
+ * the storage admits with each CTA shape (128x1, 64x2, 32x4 threads; variant 3
+ * and FP64 storage have one shape) on the lattice itself (the state is snapshot
  * and restored, so it is left unchanged) and keeps the fastest pair; ms (may
  * be NULL) receives the best time per step of variants 0..3 (0 where not run).
  * A lattice that lbm_step steps on chip is timed that way (at least 8 steps);

@@ -664,7 +664,7 @@ int lbm_tune(lbm_t h, int trial_steps, float ms[LBM_NUM_VARIANTS]) {
             continue;
         }
         float best_of_v = 1e30f;
-        const bool fixed = v == 3 || (chip && v == 0);  // one shape
+        const bool fixed = v == 3 || (chip && v == 0) || h->store == LBM_F64;  // one shape
         const int count = chip && v == 0 ? std::max(steps, lbm::kResidentMinSteps) : steps;
         for (int wi = 0; wi < (fixed ? 1 : 3) && e == cudaSuccess; ++wi) {
             h->a.variant = v;

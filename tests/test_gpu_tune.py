@@ -27,8 +27,18 @@ def test_tuning_keeps_a_small_lattice_on_chip(shape, store, trial):
         assert all((ms[v] > 0) == (v in admitted) for v in range(lbm.NUM_VARIANTS))
         if fits:  # one kernel, one time for the variants that step on chip; variant 1 launches every step
             assert len({ms[v] for v in admitted if v != 1}) == 1
-            assert L.info()["variant"] == 0
+            assert L.info()["variant"] == 0 or trial == 1  # two trial steps of variant 1 are mostly launch
         ref.set_variant(L.info()["variant"])
         L.step(40)
         ref.step(40)
         np.testing.assert_array_equal(L.get_f(), ref.get_f())
+
+
+@pytest.mark.parametrize("n", [150, 257, 400])
+def test_f64_steps_have_one_block_shape(n):
+    """The FP64 step ignores the block width: no trial of the others, and the default is kept."""
+    with lbm.Lattice(n, n, OMEGAS, store=lbm.F64) as L:
+        L.init(*workloads.random_fields(4, n, n, u_amp=0.03, rho_amp=0.01))
+        width = L.info()["block_x"]
+        assert L.tune(20)[0] > 0
+        assert L.info()["block_x"] == width
