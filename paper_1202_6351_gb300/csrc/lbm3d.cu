@@ -162,6 +162,7 @@ cudaError_t launch_step3(const Args3& a, bool odd, bool forced, cudaStream_t s) 
 int fail(int code, const char* msg) { return lbm::set_error(code, "%s", msg); }
 
 int cuda_fail(cudaError_t e, const char* what) {
+    cudaGetLastError();  // reported here: not found again by a later launch check
     return lbm::set_error(e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA, "%s: %s", what,
                           cudaGetErrorString(e));
 }

@@ -441,9 +441,11 @@ extern "C" int lbm_adjoint_run_in(lbm_t h, long nsteps, long every, const double
     const cudaError_t e2 = cudaStreamSynchronize(s);  // also after a failure: nothing still uses the workspace
     if (e == cudaSuccess) e = e2;
     if (prev >= 0 && prev != h->device) cudaSetDevice(prev);
-    if (e != cudaSuccess)
+    if (e != cudaSuccess) {
+        cudaGetLastError();  // reported here: not found again by a later launch check
         return set_error(e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA, "lbm_adjoint_run: %s",
                          cudaGetErrorString(e));
+    }
     *loss = host[0];
     if (grad_omega) {
         grad_omega[0] = host[1] / 12.0;

@@ -532,12 +532,15 @@ cudaError_t release_domains(lbm_batch_s* b) {
     return e;
 }
 
-#define BATCH_CUDA(call, what)                                                              \
-    do {                                                                                    \
-        cudaError_t e_ = (call);                                                            \
-        if (e_ != cudaSuccess)                                                              \
-            return lbm::set_error(e_ == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA, \
-                                  "%s: %s", what, cudaGetErrorString(e_));                  \
+int cuda_fail(cudaError_t e, const char* what) {
+    cudaGetLastError();  // reported here: not found again by a later launch check
+    return lbm::set_error(e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA, "%s: %s", what, cudaGetErrorString(e));
+}
+
+#define BATCH_CUDA(call, what)                             \
+    do {                                                   \
+        cudaError_t e_ = (call);                           \
+        if (e_ != cudaSuccess) return cuda_fail(e_, what); \
     } while (0)
 
 struct Guard {
@@ -605,8 +608,7 @@ int lbm_batch_create(const lbm_t* lattices, int count, lbm_batch_t* out) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) {
         lbm_batch_destroy(b);
-        return lbm::set_error(e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA, "lbm_batch_create: %s",
-                              cudaGetErrorString(e));
+        return cuda_fail(e, "lbm_batch_create");
     }
     *out = b;
     return LBM_OK;
@@ -817,9 +819,7 @@ int lbm_batch_tune(lbm_batch_t b, int trial_steps, float* best_ms) {
     if (t0) cudaEventDestroy(t0);
     if (t1) cudaEventDestroy(t1);
     drop_graph(b);
-    if (e != cudaSuccess)
-        return lbm::set_error(e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA, "lbm_batch_tune: %s",
-                              cudaGetErrorString(e));
+    if (e != cudaSuccess) return cuda_fail(e, "lbm_batch_tune");
     if (best_ms) *best_ms = b->tuned_ms;
     return LBM_OK;
 }

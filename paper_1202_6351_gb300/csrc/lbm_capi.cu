@@ -33,7 +33,10 @@ int fail(int code, const char* fmt, ...) {
     return code;
 }
 
+// Also clears the runtime's record of the error: a later launch check, here or in the caller's
+// program, would take it for its own.
 int cuda_fail(cudaError_t e, const char* what) {
+    cudaGetLastError();
     return fail(e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
