@@ -7,13 +7,31 @@ body force ``force`` [2, ny, nx], with shear rate omega_4 = omega_5 =
 ``omega_shear`` and the other rates fixed.  Its backward pass returns the
 gradients the CUDA adjoint computed in the same call (reverse streaming plus
 the transposed collision, checkpoints every ``every`` steps, FP64
-accumulation).  All tensors are float64 on the current CUDA device.
+accumulation).  All tensors are float64 on the current CUDA device.  The states
+of a run may stay in PyTorch's caching allocator after the call (KEPT_PART).
 """
 from __future__ import annotations
 
 import torch
 
 from . import lbm
+
+
+# The checkpoints of a run live in PyTorch's caching allocator, on the stream the lattice runs on, if they
+# take at most this part of the device memory (4.6 of 298 GB): a training loop maps them once instead of on
+# every call (512^2, 400 steps, 1 GB: 10.9 -> 8.6 ms).  PyTorch keeps that memory until
+# torch.cuda.empty_cache(), which lbm.py calls when an allocation of the library finds no room.  Larger
+# runs, and runs that find no room in the allocator, use memory that the library maps for the call.
+KEPT_PART = 1 / 64
+
+
+def _workspace(nbytes):
+    if nbytes > KEPT_PART * torch.cuda.get_device_properties(torch.cuda.current_device()).total_memory:
+        return None
+    try:
+        return torch.empty(nbytes, dtype=torch.uint8, device="cuda")
+    except torch.cuda.OutOfMemoryError:
+        return None
 
 
 class FinalVelocityLoss(torch.autograd.Function):
@@ -25,13 +43,7 @@ class FinalVelocityLoss(torch.autograd.Function):
         stream = torch.cuda.current_stream().cuda_stream
         with lbm.Lattice(nx, ny, rates, model=lbm.CASCADED, store=store, stream=stream) as L:
             L.set_force_field(force.detach().contiguous())
-            # The checkpoints live in PyTorch's caching allocator, on the stream the lattice runs on: a training
-            # loop maps them once instead of on every call (512^2, 400 steps: 10.9 -> 8.6 ms).  Without room
-            # there the library allocates for itself, or reports that it cannot.
-            try:
-                ws = torch.empty(L.adjoint_workspace(nsteps, every), dtype=torch.uint8, device="cuda")
-            except torch.cuda.OutOfMemoryError:
-                ws = None
+            ws = _workspace(L.adjoint_workspace(nsteps, every))
             loss, gu, gf, gom = L.adjoint_run(nsteps, every, u0.detach().contiguous(), target.detach().contiguous(),
                                               workspace=ws)
         ctx.save_for_backward(gu, gf)

@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import sys
 
 import numpy as np
 
@@ -127,6 +128,19 @@ def _check(rc: int):
         raise LBMError(rc, load_library().lbm_last_error().decode())
 
 
+def _check_alloc(call, *args):
+    """A call that may allocate device memory: if there is none, once more after PyTorch's
+    caching allocator has given back what it holds unused (the autograd function of
+    adjoint.py leaves its checkpoints there)."""
+    rc = call(*args)
+    if rc == LBM_ENOMEM:
+        torch = sys.modules.get("torch")
+        if torch is not None and torch.cuda.is_initialized():
+            torch.cuda.empty_cache()
+            rc = call(*args)
+    _check(rc)
+
+
 def _darr(v, n):
     return (C.c_double * n)(*[float(x) for x in v])
 
@@ -155,8 +169,8 @@ def lbm_create(nx, ny, omegas, force=(0.0, 0.0), edges=(PERIODIC,) * 4, wall_u=(
     lib = load_library()
     bc = lbm_bc_t((C.c_int * 4)(*[int(e) for e in edges]), _darr(wall_u, 4))
     h = C.c_void_p()
-    _check(lib.lbm_create(int(nx), int(ny), _darr(omegas, 6), _darr(force, 2), C.byref(bc), int(model),
-                          int(store), float(rho0), C.byref(h)))
+    _check_alloc(lib.lbm_create, int(nx), int(ny), _darr(omegas, 6), _darr(force, 2), C.byref(bc), int(model),
+                          int(store), float(rho0), C.byref(h))
     return h
 
 
@@ -262,7 +276,7 @@ class Lattice:
         return self
 
     def set_variant(self, variant):
-        _check(self.lib.lbm_set_variant(self.h, int(variant)))
+        _check_alloc(self.lib.lbm_set_variant, self.h, int(variant))
         return self
 
     def set_rounding(self, mode, seed=0):
@@ -274,7 +288,7 @@ class Lattice:
         """Time the kernel variants and CTA shapes, keep the fastest; returns the
         best ms per step of variants 0..3 (0.0 where the storage has no such variant)."""
         ms = (C.c_float * NUM_VARIANTS)()
-        _check(self.lib.lbm_tune(self.h, int(trial_steps), ms))
+        _check_alloc(self.lib.lbm_tune, self.h, int(trial_steps), ms)
         return tuple(ms)
 
     def set_force_field(self, fxy):
@@ -285,12 +299,12 @@ class Lattice:
             import torch
 
             if isinstance(fxy, torch.Tensor):
-                _check(self.lib.lbm_set_force_field(self.h, _dev(fxy, (2,) + self.shape), 1))
+                _check_alloc(self.lib.lbm_set_force_field, self.h, _dev(fxy, (2,) + self.shape), 1)
                 return
         except ImportError:
             pass
         a, p = _host(fxy, (2,) + self.shape)
-        _check(self.lib.lbm_set_force_field(self.h, p, 0))
+        _check_alloc(self.lib.lbm_set_force_field, self.h, p, 0)
 
     def init(self, rho=None, u=None):
         ra = ua = None
@@ -299,7 +313,7 @@ class Lattice:
             ra, rp = _host(rho, self.shape)
         if u is not None:
             ua, up = _host(u, (2,) + self.shape)
-        _check(self.lib.lbm_init(self.h, rp, up))
+        _check_alloc(self.lib.lbm_init, self.h, rp, up)
         return self
 
     def init_device(self, rho=None, u=None):
@@ -315,7 +329,7 @@ class Lattice:
     def macros(self):
         rho = np.empty(self.shape)
         u = np.empty((2,) + self.shape)
-        _check(self.lib.lbm_macros(self.h, rho.ctypes.data, u.ctypes.data))
+        _check_alloc(self.lib.lbm_macros, self.h, rho.ctypes.data, u.ctypes.data)
         return rho, u
 
     def macros_device(self, rho=None, u=None):
@@ -328,17 +342,17 @@ class Lattice:
 
     def strain(self):
         out = np.empty((3,) + self.shape)
-        _check(self.lib.lbm_strain(self.h, out.ctypes.data))
+        _check_alloc(self.lib.lbm_strain, self.h, out.ctypes.data)
         return out
 
     def get_f(self):
         f = np.empty((9,) + self.shape)
-        _check(self.lib.lbm_get_f(self.h, f.ctypes.data))
+        _check_alloc(self.lib.lbm_get_f, self.h, f.ctypes.data)
         return f
 
     def set_f(self, f):
         a, p = _host(f, (9,) + self.shape)
-        _check(self.lib.lbm_set_f(self.h, p))
+        _check_alloc(self.lib.lbm_set_f, self.h, p)
         return self
 
     def get_f_device(self, out=None):
@@ -383,10 +397,10 @@ class Lattice:
             if not (workspace.is_cuda and workspace.is_contiguous()):
                 raise TypeError("workspace: expected a contiguous CUDA tensor")
             ws, nbytes = workspace.data_ptr(), workspace.numel() * workspace.element_size()
-        _check(self.lib.lbm_adjoint_run_in(
+        _check_alloc(self.lib.lbm_adjoint_run_in,
             self.h, int(nsteps), int(every), _dev(rho, self.shape) if rho is not None else None,
             _dev(u0, shape2), _dev(u_target, shape2), C.byref(loss),
-            gu.data_ptr() if gu is not None else None, gf.data_ptr() if gf is not None else None, gom, ws, nbytes))
+            gu.data_ptr() if gu is not None else None, gf.data_ptr() if gf is not None else None, gom, ws, nbytes)
         return loss.value, gu, gf, np.array(list(gom))
 
 
@@ -404,7 +418,7 @@ class Batch:
         arr = (C.c_void_p * len(self.lattices))(*[L.h.value if isinstance(L.h, C.c_void_p) else L.h
                                                    for L in self.lattices])
         self.b = C.c_void_p()
-        _check(self.lib.lbm_batch_create(arr, len(self.lattices), C.byref(self.b)))
+        _check_alloc(self.lib.lbm_batch_create, arr, len(self.lattices), C.byref(self.b))
 
     def close(self):
         b, self.b = self.b, None
@@ -426,7 +440,7 @@ class Batch:
 
     def tune(self, trial_steps=5):
         ms = C.c_float()
-        _check(self.lib.lbm_batch_tune(self.b, int(trial_steps), C.byref(ms)))
+        _check_alloc(self.lib.lbm_batch_tune, self.b, int(trial_steps), C.byref(ms))
         return ms.value
 
     def step(self, n=1):
@@ -438,7 +452,7 @@ class Batch:
 
     def set_two_step(self, on=True):
         """Two steps per launch for the whole batch (lbm_batch_set_two_step)."""
-        _check(self.lib.lbm_batch_set_two_step(self.b, 1 if on else 0))
+        _check_alloc(self.lib.lbm_batch_set_two_step, self.b, 1 if on else 0)
         return self
 
     def sync(self):
@@ -463,8 +477,8 @@ class Lattice3:
         self.shape = (int(nz), int(ny), int(nx))
         self.store = int(store)
         h = C.c_void_p()
-        _check(self.lib.lbm3_create(int(nx), int(ny), int(nz), _darr(omegas, 6), _darr(force, 3), int(store),
-                                    float(rho0), C.byref(h)))
+        _check_alloc(self.lib.lbm3_create, int(nx), int(ny), int(nz), _darr(omegas, 6), _darr(force, 3), int(store),
+                                    float(rho0), C.byref(h))
         self.h = h
         if stream is not None:
             _check(self.lib.lbm3_set_stream(self.h, C.c_void_p(stream)))
@@ -497,7 +511,7 @@ class Lattice3:
             ra, rp = _host(rho, self.shape)
         if u is not None:
             ua, up = _host(u, (3,) + self.shape)
-        _check(self.lib.lbm3_init(self.h, rp, up))
+        _check_alloc(self.lib.lbm3_init, self.h, rp, up)
         return self
 
     def step(self, n=1):
@@ -507,17 +521,17 @@ class Lattice3:
     def macros(self):
         rho = np.empty(self.shape)
         u = np.empty((3,) + self.shape)
-        _check(self.lib.lbm3_macros(self.h, rho.ctypes.data, u.ctypes.data))
+        _check_alloc(self.lib.lbm3_macros, self.h, rho.ctypes.data, u.ctypes.data)
         return rho, u
 
     def get_f(self):
         f = np.empty((27,) + self.shape)
-        _check(self.lib.lbm3_get_f(self.h, f.ctypes.data))
+        _check_alloc(self.lib.lbm3_get_f, self.h, f.ctypes.data)
         return f
 
     def set_f(self, f):
         a, p = _host(f, (27,) + self.shape)
-        _check(self.lib.lbm3_set_f(self.h, p))
+        _check_alloc(self.lib.lbm3_set_f, self.h, p)
         return self
 
     def info(self):

@@ -30,3 +30,19 @@ def test_a_refused_allocation_is_not_reported_by_later_calls():
         finally:
             for h in held:
                 h.close()
+
+
+def test_memory_that_pytorch_holds_unused_is_given_back():
+    """PyTorch's caching allocator keeps freed tensors; a lattice that needs their memory gets it."""
+    import torch
+
+    torch.cuda.empty_cache()
+    total = torch.cuda.get_device_properties(0).total_memory
+    block = torch.empty(int(total * 0.55), dtype=torch.uint8, device="cuda")
+    del block
+    assert torch.cuda.memory_reserved() > 0.5 * total
+    try:
+        with lbm.Lattice(*HUGE, OMEGAS, store=lbm.F64) as L:
+            assert L.time == 0
+    finally:
+        torch.cuda.empty_cache()
