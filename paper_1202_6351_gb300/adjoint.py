@@ -18,11 +18,12 @@ from . import lbm
 
 
 # The checkpoints of a run live in PyTorch's caching allocator, on the stream the lattice runs on, if they
-# take at most this part of the device memory (4.6 of 298 GB): a training loop maps them once instead of on
-# every call (512^2, 400 steps, 1 GB: 10.9 -> 8.6 ms).  PyTorch keeps that memory until
-# torch.cuda.empty_cache(), which lbm.py calls when an allocation of the library finds no room.  Larger
-# runs, and runs that find no room in the allocator, use memory that the library maps for the call.
-KEPT_PART = 1 / 64
+# take at most this part of the device memory (18.6 of 298 GB): a training loop maps them once instead of on
+# every call (ms per call mapped on each call -> kept: 512^2, 400 steps, 1.0 GB 10.6 -> 8.4; 2048^2, 100 steps,
+# 4.0 GB 35.2 -> 27.0, 15.5 GB 58.4 -> 27.3).  PyTorch keeps that memory until torch.cuda.empty_cache(), which
+# lbm.py calls when an allocation of the library finds no room.  Larger runs, and runs that find no room in
+# the allocator, use memory that the library maps for the call.
+KEPT_PART = 1 / 16
 
 
 def _workspace(nbytes):
