@@ -34,8 +34,14 @@
 //
 // A lattice of fewer than kMultiSmallNodes nodes has too few such tiles to fill the
 // SMs: 32 x 16 tiles there, loaded by every thread (most are edge tiles, which
-// a tensor copy would have to patch): FP32 257^2 2.1 us per step against 3.5 with
-// the two-step kernel.
+// a tensor copy would have to patch).  us per step of 32 x 16 tiles | 56 x 40 tiles | the
+// two-step kernel: FP32 257^2 1.89 | 3.81 | 3.46, 384^2 2.47 | 3.59 | 3.45, 480^2 3.10 | 3.57,
+// 512^2 4.13 | 3.56 | 4.56, 560^2 4.89 | 3.67, 600^2 5.10 | 5.28 | 5.53, 640^2 5.58 | 5.38, 700^2
+// 6.37 | 5.76 | 6.60; FP16 480^2 3.17 | 3.57, 560^2 4.80 | 3.64, 600^2 5.00 | 5.29, 640^2 5.68 |
+// 5.45.  Both go in waves of blocks (32 x 16: 456 at a time; 56 x 40: 152 alone on their SM,
+// then two), so the better one changes twice between 480^2 and 640^2; the line is the last
+// crossing.  One step per launch (variant 0) beats both on these lattices: FP32 257^2
+// 1.70, 384^2 2.18, 512^2 3.18, 600^2 3.92, 700^2 4.91.
 #pragma once
 
 #include <cuda.h>
