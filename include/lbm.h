@@ -270,8 +270,8 @@ size_t lbm_bytes_per_update(int store);
  * state is copied; every = 1 keeps every state and recomputes nothing.
  * Device memory used during the call: (ceil(nsteps/every) +
  * max(1, min(every, nsteps) - 1)) times the population array, two adjoint
- * arrays, a force-gradient array, its FP32 segment sum (FP32 storage) and small
- * scratch, allocated and released in stream order.  Synchronous.
+ * arrays, a force-gradient array if grad_force is NULL, its FP32 segment sum
+ * (FP32 storage) and small scratch, allocated and released in stream order.  Synchronous.
  * Leaves the lattice at step nsteps. */
 int lbm_adjoint_run(lbm_t h, long nsteps, long every, const double* rho, const double* u0, const double* u_target,
                     double* loss, double* grad_u0, double* grad_force, double grad_omega[6]);

@@ -361,8 +361,8 @@ struct AdjointSpace {
         acc = take(7 * sizeof(double));
         gc = take(6 * lbm::adj_slots(h->a) * sizeof(double));
         lossp = take(((size_t)h->a.nx + lbm::kThreads - 1) / lbm::kThreads * h->a.ny * sizeof(double));
-        gF = take(2 * n * sizeof(double));
         gseg = take(dbl ? 0 : 2 * n * sizeof(float));
+        gF = take(2 * n * sizeof(double));  // last: a run that is given the array does not need it
     }
 };
 
@@ -414,10 +414,11 @@ extern "C" int lbm_adjoint_run_in(lbm_t h, long nsteps, long every, const double
     if (prev != h->device) cudaSetDevice(h->device);
     cudaStream_t s = h->stream;
     char* space = static_cast<char*>(workspace);
-    if (!space && cudaMallocAsync((void**)&space, at.total, s) != cudaSuccess) {
+    const size_t own = grad_force ? at.gF : at.total;
+    if (!space && cudaMallocAsync((void**)&space, own, s) != cudaSuccess) {
         cudaGetLastError();
         if (prev >= 0 && prev != h->device) cudaSetDevice(prev);
-        return set_error(LBM_ENOMEM, "lbm_adjoint_run: cannot allocate %.1f MB of checkpoints and buffers", at.total / 1e6);
+        return set_error(LBM_ENOMEM, "lbm_adjoint_run: cannot allocate %.1f MB of checkpoints and buffers", own / 1e6);
     }
     char* ckpt = space + at.ckpt;
     char* seg = space + at.seg;
