@@ -170,7 +170,7 @@ def lbm_create(nx, ny, omegas, force=(0.0, 0.0), edges=(PERIODIC,) * 4, wall_u=(
     bc = lbm_bc_t((C.c_int * 4)(*[int(e) for e in edges]), _darr(wall_u, 4))
     h = C.c_void_p()
     _check_alloc(lib.lbm_create, int(nx), int(ny), _darr(omegas, 6), _darr(force, 2), C.byref(bc), int(model),
-                          int(store), float(rho0), C.byref(h))
+                 int(store), float(rho0), C.byref(h))
     return h
 
 
@@ -383,24 +383,26 @@ class Lattice:
 
     def adjoint_run(self, nsteps, every, u0, u_target, rho=None, want_u0=True, want_force=True, workspace=None):
         """lbm_adjoint_run with float64 CUDA tensors; returns (loss, grad_u0, grad_force, grad_omega[6]).
-        workspace: a contiguous CUDA tensor of at least adjoint_workspace(nsteps, every) bytes to run in
-        (lbm_adjoint_run_in), or None to allocate it for the call."""
+        workspace: a contiguous CUDA tensor of at least adjoint_workspace(nsteps, every) bytes on the device
+        of u0 to run in (lbm_adjoint_run_in), or None to allocate it for the call."""
         import torch
 
         shape2 = (2,) + self.shape
         gu = torch.empty(shape2, dtype=torch.float64, device="cuda") if want_u0 else None
         gf = torch.empty(shape2, dtype=torch.float64, device="cuda") if want_force else None
+        pu0, pt = _dev(u0, shape2), _dev(u_target, shape2)
         loss = C.c_double()
         gom = (C.c_double * 6)()
         ws, nbytes = None, 0
         if workspace is not None:
             if not (workspace.is_cuda and workspace.is_contiguous()):
                 raise TypeError("workspace: expected a contiguous CUDA tensor")
+            if workspace.device != u0.device:
+                raise ValueError(f"workspace: expected on {u0.device}, the device of u0, not on {workspace.device}")
             ws, nbytes = workspace.data_ptr(), workspace.numel() * workspace.element_size()
-        _check_alloc(self.lib.lbm_adjoint_run_in,
-            self.h, int(nsteps), int(every), _dev(rho, self.shape) if rho is not None else None,
-            _dev(u0, shape2), _dev(u_target, shape2), C.byref(loss),
-            gu.data_ptr() if gu is not None else None, gf.data_ptr() if gf is not None else None, gom, ws, nbytes)
+        _check_alloc(self.lib.lbm_adjoint_run_in, self.h, int(nsteps), int(every),
+                     _dev(rho, self.shape) if rho is not None else None, pu0, pt, C.byref(loss),
+                     gu.data_ptr() if gu is not None else None, gf.data_ptr() if gf is not None else None, gom, ws, nbytes)
         return loss.value, gu, gf, np.array(list(gom))
 
 
@@ -478,7 +480,7 @@ class Lattice3:
         self.store = int(store)
         h = C.c_void_p()
         _check_alloc(self.lib.lbm3_create, int(nx), int(ny), int(nz), _darr(omegas, 6), _darr(force, 3), int(store),
-                                    float(rho0), C.byref(h))
+                     float(rho0), C.byref(h))
         self.h = h
         if stream is not None:
             _check(self.lib.lbm3_set_stream(self.h, C.c_void_p(stream)))
