@@ -701,7 +701,7 @@ int lbm_batch_sync(lbm_batch_t b) {
         BATCH_CUDA(cudaMemcpy(&v, b->d_err, sizeof(int), cudaMemcpyDeviceToHost), "lbm_batch_sync: error word");
         if (v) {
             cudaMemset(b->d_err, 0, sizeof(int));
-            return fail(LBM_ECUDA, "lbm_batch_sync: a two-step launch timed out waiting for its tile load");
+            return fail(LBM_ECUDA, "lbm_batch_sync: a launch of several steps timed out waiting for its tile load");
         }
     }
     return LBM_OK;

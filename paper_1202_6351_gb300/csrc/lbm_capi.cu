@@ -259,7 +259,7 @@ int fused_error(lbm_s* h) {
     if (cudaMemcpy(&v, h->d_err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return LBM_ECUDA;
     if (v == 0) return LBM_OK;
     cudaMemset(h->d_err, 0, sizeof(int));
-    return lbm::set_error(LBM_ECUDA, "a fused two-step launch timed out waiting for its tile load; the state is invalid");
+    return lbm::set_error(LBM_ECUDA, "a launch of several steps (variant 3) timed out waiting for its tile load; the state is invalid");
 }
 
 // Steps per graph replay: a multiple of 4 with fused steps (an even number of
