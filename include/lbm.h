@@ -188,10 +188,12 @@ int lbm_init_device(lbm_t h, const double* rho, const double* u);
 
 /* Advance n >= 0 time steps (collide Eq. 23 + stream Eq. 24 per step), one
  * fused kernel launch per step (several with variant 3), asynchronously on the
- * handle's stream.  Small lattices (LBM_F32, LBM_BF16DEV, LBM_F16DEV; up to
- * 16 x 800 nodes, with a sixteenth of the rows, rounded up, of at most 800 nodes;
- * every variant but 1) take 8 or more steps in one launch of a kernel that keeps
- * the lattice in the shared memory of one thread-block cluster; the results are
+ * handle's stream.  Small lattices take 8 or more steps of a call in one launch
+ * of a kernel that keeps the lattice in the shared memory of one thread-block
+ * cluster (every variant but 1): those of which a sixteenth of the rows, rounded
+ * up, has at most 800 nodes (a lattice of fewer than 16 rows is cut into 8, 4, 2
+ * or 1 parts); at most 720 with a force or stochastic rounding, 512
+ * with both in LBM_F32, 128 for LBM_F64.  The results are
  * bit for bit those of variants 0, 2 and 3.  Elsewhere runs
  * of at least lbm_set_graph_steps steps starting at an even step are replayed
  * from a CUDA graph on an internal stream that is ordered after the handle's

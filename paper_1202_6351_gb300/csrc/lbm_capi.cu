@@ -316,7 +316,7 @@ cudaError_t launch_resident(const lbm_s* h, long t0, int n) {
 // Small lattices step on chip, whatever the variant (the results are
 // those of variants 0, 2 and 3); variant 1, which rounds differently, stays itself.
 bool resident_active(lbm_s* h) {
-    if (h->a.variant == 1 || !lbm::resident_fits(h->a, h->store)) return false;
+    if (h->a.variant == 1 || !lbm::resident_fits(h->a, h->store, force_mode(h))) return false;
     if (h->resident < 0) {
         h->resident = launch_resident(h, h->t, 0) == cudaSuccess ? 1 : 0;
         if (!h->resident) cudaGetLastError();

@@ -14,8 +14,9 @@
 // A step costs about 0.4 us of latency (barrier, loads, the collision's chain) plus
 // instruction issue of five warps per SM quarter at most, so the lattice is spread
 // over as many CTAs as a cluster takes (64^2 cavity: 0.87 us with 8, 0.69 with 16).
-// Beyond one node per thread (800 a CTA, 80 registers each) a launch per step over
-// all 152 SMs wins: 128^2 1.8 us here with two rounds, 1.5 there.  An FP64 step costs its
+// Beyond one node per thread (800 a CTA, 80 registers each; fewer for the longer
+// updates, resident_nodes) a launch per step over all 152 SMs wins: 128^2 1.8 us here
+// with two rounds, 1.5 there.  An FP64 step costs its
 // instructions (64 cycles each per warp and SM quarter), so beyond 128 nodes a CTA,
 // one warp per quarter, the launch over all SMs wins; up to there what is saved is
 // the launch and the filling of the chip.
@@ -43,9 +44,24 @@ inline int resident_size(const Args& a) {
     while (size > a.ny) size /= 2;
     return size;
 }
-inline bool resident_fits(const Args& a, int store) {
+// Most nodes of a CTA with which the steps on chip are no slower than a launch per step: a
+// step costs its instructions on 16 SMs, so a force and stochastic rounding lower the
+// line.  Speed of 512 steps on chip over 64-step graph replays, over the three
+// collisions, periodic and cavity, with 16 or more rows (the lower end: slabs of one row):
+//   FP32 stochastic, forced   480 nodes 0.96-1.36, 560 0.93-1.27, 707 0.88-1.05, 800 0.68-0.93
+//   FP32 stochastic           640 1.04-1.31, 707 1.12-1.20, 784 0.94-1.11, 800 0.84-1.06
+//   forced, FP32 and 16-bit   707 1.04-1.52, 784 0.94-1.25, 800 0.79-1.26
+//   neither                   707 1.38-1.71, 784 1.26-1.54, 800 0.95-1.55
+//   FP64                      128 0.99-1.3
+// (112^2 FP32 stochastic with a force field: 2.15 us per step on chip, 1.67 launched.)
+inline int resident_nodes(int store, int force, bool stochastic) {
+    if (store == LBM_F64) return resident_threads(store);
+    if (store == LBM_F32 && stochastic && force != 0) return 512;
+    return force != 0 || stochastic ? 720 : resident_threads(store);
+}
+inline bool resident_fits(const Args& a, int store, int force) {
     const int size = resident_size(a);
-    return (long long)((a.ny + size - 1) / size) * a.nx <= resident_threads(store);
+    return (long long)((a.ny + size - 1) / size) * a.nx <= resident_nodes(store, force, a.rseed != 0);
 }
 
 __device__ __forceinline__ unsigned cluster_rank() {
