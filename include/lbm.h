@@ -119,10 +119,11 @@ int lbm_set_omegas(lbm_t h, const double omegas[6]);
  * (temporal blocking): a CTA loads a tile of nodes with its halo into shared
  * memory, takes the steps there and writes the tile once, so the populations
  * cross HBM once per launch.  The cascaded collision without a force and with
- * round to nearest takes four steps per launch (56 x 40 tiles; 32 x 16 below
- * 360,000 nodes), everything else two (64 x 16 tiles).  Variant 3 keeps a second
- * population array (ping-pong, allocated by this call; LBM_ENOMEM if it does not
- * fit), starts a launch at even steps, takes what is left over in single steps
+ * round to nearest takes four steps per launch (56 x 40 tiles, or 32 x 16 where
+ * those are estimated to be faster: small and narrow lattices) and two for a
+ * remainder of two or three, everything else two (64 x 16 tiles).  Variant 3 keeps a
+ * second population array (ping-pong, allocated by this call; LBM_ENOMEM if it does
+ * not fit), starts a launch at even steps, takes what is left over in single steps
  * (variant 2 for 16-bit stores, else 0), needs a lattice of at
  * least 4 x 4 nodes and is not used while the divergence check is on.
  * The default is 2 for 16-bit stores of at least 2^20 nodes and 0

@@ -32,16 +32,21 @@
 // (64 x 32); the two-step kernel 138.7.  FP16: 56 x 40 with three CTAs 175.9, two
 // 163.8, 128 x 32 177.3; two-step kernel 135.9, four nodes per thread 152.8.
 //
-// A lattice of fewer than kMultiSmallNodes nodes has too few such tiles to fill the
-// SMs: 32 x 16 tiles there, loaded by every thread (most are edge tiles, which
-// a tensor copy would have to patch).  us per step of 32 x 16 tiles | 56 x 40 tiles | the
-// two-step kernel: FP32 257^2 1.89 | 3.81 | 3.46, 384^2 2.47 | 3.59 | 3.45, 480^2 3.10 | 3.57,
-// 512^2 4.13 | 3.56 | 4.56, 560^2 4.89 | 3.67, 600^2 5.10 | 5.28 | 5.53, 640^2 5.58 | 5.38, 700^2
-// 6.37 | 5.76 | 6.60; FP16 480^2 3.17 | 3.57, 560^2 4.80 | 3.64, 600^2 5.00 | 5.29, 640^2 5.68 |
-// 5.45.  Both go in waves of blocks (32 x 16: 456 at a time; 56 x 40: 152 alone on their SM,
-// then two), so the better one changes twice between 480^2 and 640^2; the line is the last
-// crossing.  One step per launch (variant 0) beats both on these lattices: FP32 257^2
-// 1.70, 384^2 2.18, 512^2 3.18, 600^2 3.92, 700^2 4.91.
+// Few such tiles do not fill the SMs, and a row of them with one ragged column puts the
+// full ones on every other SM.  Then 32 x 16 tiles, loaded by every thread (most are edge
+// tiles, which a tensor copy would have to patch).  us per step of 32 x 16 tiles | 56 x 40
+// tiles | the two-step kernel: FP32 257^2 1.89 | 3.81 | 3.46, 384^2 2.47 | 3.59 | 3.45, 480^2
+// 3.10 | 3.57, 512^2 4.13 | 3.56 | 4.56, 560^2 4.89 | 3.67, 600^2 5.10 | 5.28 | 5.53, 640^2
+// 5.58 | 5.38, 700^2 6.37 | 5.76 | 6.60, 57 x 8000 6.42 | 9.01 | 7.34, 20 x 20000 6.64 | 11.77 |
+// 13.2; FP16 480^2 3.17 | 3.57, 560^2 4.80 | 3.64, 600^2 5.00 | 5.29, 640^2 5.68 | 5.45.  Both go in
+// waves of blocks (456 of the small; 152 alone on their SM, then 304 of the large), so
+// multi_small_us and multi_large_us are what was measured, by number of tiles, and
+// the smaller one wins.  One step per launch (variant 0) beats both below about 750^2:
+// FP32 257^2 1.70, 384^2 2.18, 512^2 3.18, 600^2 3.92, 700^2 4.91.
+//
+// Up to two 56 x 40 tiles per SM (304) the third block that 16-bit storage has room for stays
+// unused: 384 threads a block then, as for FP32 (FP16 640^2 5.47 -> 5.25, 560^2 3.64 ->
+// 3.37, 1000 x 401 5.51 -> 5.34; the two-step kernel 5.33, 5.36, 5.33).
 #pragma once
 
 #include <cuda.h>
@@ -54,7 +59,6 @@
 namespace lbm {
 
 constexpr int kMultiSteps = 4;  // halo of the shared-memory box, the most steps of a launch
-constexpr long long kMultiSmallNodes = 600LL * 600;
 
 template <int STORE_, int TX_, int TY_, int NT_, int MINB_, bool TMA_>
 struct MultiGeom {
@@ -72,6 +76,7 @@ struct MultiGeom {
 };
 template <int STORE> struct MultiLarge : MultiGeom<STORE, 56, 40, 256, 3, true> {};
 template <> struct MultiLarge<LBM_F32> : MultiGeom<LBM_F32, 56, 40, 384, 2, true> {};
+template <int STORE> struct MultiWide : MultiGeom<STORE, 56, 40, 384, 2, true> {};
 template <int STORE> struct MultiSmall : MultiGeom<STORE, 32, 16, 256, 3, false> {};
 
 enum : int { kMultiErrTimeout = 1 };
@@ -376,11 +381,29 @@ static cudaError_t launch_multi_geom(const CUtensorMap& map, const Args& a, void
                         s, map, a, static_cast<const void*>(a.f), out, err, steps);
 }
 
+// us per step of n tiles of 32 x 16 and of n full tiles of 56 x 40 nodes, FP32, as measured
+// (above); a lattice without walls has more halo to patch.
+inline double multi_small_us(double n) {
+    return n <= 152 ? 1.9 : n <= 304 ? 2.5 : n <= 456 ? 3.1 : n <= 554 ? 4.1 : 1.0 + 0.0056 * n;
+}
+inline double multi_large_us(double n, bool walls) {
+    return n <= 152 ? 3.6 : n <= 304 ? (walls ? 5.2 : 5.4) : 2.4 + 0.0132 * n;
+}
+
 template <int STORE>
 static cudaError_t launch_multi_store(const CUtensorMap& map, const Args& a, void* out, int* err, int steps,
                                       cudaStream_t s) {
-    if ((long long)a.nx * a.ny < kMultiSmallNodes) return launch_multi_geom<MultiSmall<STORE>>(map, a, out, err, steps, s);
-    return launch_multi_geom<MultiLarge<STORE>>(map, a, out, err, steps, s);
+    using Large = MultiLarge<STORE>;
+    using Small = MultiSmall<STORE>;
+    const int gx = (a.nx + Large::TX - 1) / Large::TX, gy = (a.ny + Large::TY - 1) / Large::TY;
+    const double full = gx * (a.ny + 5.0 * gy) / (Large::TY + 5);  // a tile costs its rows plus five, whatever its width
+    const double small = double((a.nx + Small::TX - 1) / Small::TX) * ((a.ny + Small::TY - 1) / Small::TY);
+    if (multi_small_us(small) < multi_large_us(full, a.wall[LBM_WEST] || a.wall[LBM_SOUTH]))
+        return launch_multi_geom<Small>(map, a, out, err, steps, s);
+    if constexpr (STORE != LBM_F32) {
+        if ((long long)gx * gy <= 304) return launch_multi_geom<MultiWide<STORE>>(map, a, out, err, steps, s);
+    }
+    return launch_multi_geom<Large>(map, a, out, err, steps, s);
 }
 
 }  // namespace lbm
