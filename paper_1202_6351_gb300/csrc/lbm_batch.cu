@@ -292,11 +292,35 @@ void tiles2_of(const lbm_s* h, bool multi, int* tx, int* ty) {
     *ty = (h->a.ny + TY - 1) / TY;
 }
 
+// Multi-step tiles of all lattices.
+long long multi_tiles_of(const lbm_batch_s* b) {
+    long long n = 0;
+    for (const lbm_s* h : b->doms) {
+        int tx, ty;
+        tiles2_of(h, true, &tx, &ty);
+        n += (long long)tx * ty;
+    }
+    return n;
+}
+
+// Whether the batch takes the multi-step tiles: every lattice admits them, and they are one
+// per SM at most (then a launch costs its latency) or cost less in sum.  In rows of node
+// pairs, a multi-step tile costs its rows plus five whatever its width, a quarter more on a
+// periodic lattice (halo cells fetched one by one), and a two-step tile 39.8.  us per step, two
+// steps per launch | four, FP32 periodic: 200 x 57^2 11.5 | 13.5, 64^2 11.3 | 13.4, 72^2 24.5 | 15.1, 128^2
+// 42.5 | 35.5; 60 x 64^2 5.3 | 6.1; 4 x 64^2 4.7 | 4.4; 200 cavities of 57^2 12.2 | 12.9, 64^2 12.3 | 12.4.
 bool multi_admitted(const lbm_batch_s* b) {
     if (b->model != LBM_CASCADED) return false;
-    for (const lbm_s* h : b->doms)
+    double multi = 0.0, two = 0.0;
+    for (const lbm_s* h : b->doms) {
         if (lbm::force_mode(h) != 0 || h->a.rseed != 0) return false;
-    return true;
+        int mx, my, tx, ty;
+        tiles2_of(h, true, &mx, &my);
+        tiles2_of(h, false, &tx, &ty);
+        multi += (h->walls ? 1.0 : 1.25) * mx * (h->a.ny + 5.0 * my);
+        two += 39.8 * tx * ty;
+    }
+    return multi_tiles_of(b) <= b->sms || multi <= two;
 }
 
 // The tiles of every lattice into dt, ordered by class and within a class
@@ -311,15 +335,30 @@ cudaError_t order_tiles2(lbm_batch_s* b, int* dt) {
     std::stable_sort(idx.begin(), idx.end(), [&](int p, int q) {
         return cls[p] != cls[q] ? cls[p] < cls[q] : nodes(p) > nodes(q);
     });
-    std::vector<int> t;
+    // Blocks are placed in the order of the list, a block per SM at a time: many lattices of one
+    // size would give one SM only full tiles and the next only ragged ones.  With few tiles
+    // per SM the tallest go first (200 x 48^2 FP32 8.9 -> 7.2 us per step, 60 x 57^2 cavities 6.1 ->
+    // 4.8, 60 x 128^2 12.5 -> 10.9; 200 x 72^2 FP16 13.1 -> 13.5); with many it evens out by itself, and
+    // neighbouring tiles are better taken together (200 x 256^2 98 us, 102 sorted).
+    const long long total = multi ? multi_tiles_of(b) : 0;
+    const bool by_rows = total > b->sms && total <= 8LL * b->sms;
+    struct Tile { int d, i, j, rows; };
+    std::vector<Tile> tiles;
     int first[lbm::kBatchClasses + 1] = {};
     for (int d : idx) {
+        const lbm_s* h = b->doms[d];
         int tx, ty;
-        tiles2_of(b->doms[d], multi, &tx, &ty);
+        tiles2_of(h, multi, &tx, &ty);
         for (int j = 0; j < ty; ++j)
-            for (int i = 0; i < tx; ++i) t.insert(t.end(), {d, i, j});
+            for (int i = 0; i < tx; ++i) tiles.push_back({d, i, j, std::min(MultiTile::TY, h->a.ny - j * MultiTile::TY)});
         first[cls[d] + 1] += tx * ty;
     }
+    if (by_rows)
+        std::stable_sort(tiles.begin(), tiles.end(), [&](const Tile& p, const Tile& q) {
+            return cls[p.d] != cls[q.d] ? cls[p.d] < cls[q.d] : p.rows > q.rows;
+        });
+    std::vector<int> t;
+    for (const Tile& k : tiles) t.insert(t.end(), {k.d, k.i, k.j});
     int present = 0;
     for (int c = 0; c < lbm::kBatchClasses; ++c) {
         present += first[c + 1] > 0;
