@@ -670,7 +670,7 @@ def run_batch_extras(lbm, torch, np, peak, sp, steps=200, count=96):
     """Batched ensemble: 96 domains (sides log-uniform in [64, 2048], half
     lid-driven cavities at Re in [100, 5000], half Taylor-Green, FP32 / FP16
     storage), advanced together in the configuration the batch tuner keeps (one
-    launch per step over all tiles, or one launch per two steps with a kernel
+    launch per step over all tiles, or one launch per two or four steps with a kernel
     per class of lattice) under CUDA graphs of 100 steps, against one lbm_step
     launch per domain per step."""
     from paper_1202_6351_gb300 import workloads

@@ -205,7 +205,9 @@ int lbm_init_device(lbm_t h, const double* rho, const double* u);
  * check and returns LBM_EDIVERGED when it fails. */
 int lbm_step(lbm_t h, long n);
 
-/* Steps per CUDA-graph replay in lbm_step (even; 0 disables graphs; default 64). */
+/* Steps per CUDA-graph replay in lbm_step (even; 0 disables graphs; default 64).
+ * Launches of four steps (variant 3) are queued one by one and steps on chip are
+ * one launch: neither uses a graph. */
 int lbm_set_graph_steps(lbm_t h, int steps);
 
 /* Density [ny][nx] and velocity [2][ny][nx] of Eq. (26)-(27) at the current
@@ -295,8 +297,8 @@ int lbm_adjoint_run_in(lbm_t h, long nsteps, long every, const double* rho, cons
 /* ---------------------------------------------------------------------------
  * Batches: many independent lattices advanced together (no counterpart in the
  * paper).  One time step of every lattice in the batch is ONE launch of a
- * kernel whose CTAs walk a work list of (lattice, tile) items, or two steps
- * are one launch per class of lattice (lbm_batch_set_two_step); the per-node
+ * kernel whose CTAs walk a work list of (lattice, tile) items, or two or four
+ * steps are one launch per class of lattice (lbm_batch_set_two_step); the per-node
  * update is exactly that of lbm_step, so results are bitwise equal.
  * Chunks of `graph_steps` steps (default 100, even) are replayed from a CUDA
  * graph.  All lattices must share the device and the collision model, use
@@ -321,8 +323,8 @@ int lbm_batch_destroy(lbm_batch_t b);
  * largest first; or one tile of each lattice in turn) and scheduling policy
  * (a resident grid walking the list round robin, in contiguous chunks or
  * dynamically via an atomic counter; or one CTA per tile), and, where every
- * lattice admits it and all are at the same even step, two steps per launch
- * (lbm_batch_set_two_step); keeps the fastest.  The lattices' states are
+ * lattice admits it and all are at the same even step, two or four steps per
+ * launch (lbm_batch_set_two_step); keeps the fastest.  The lattices' states are
  * snapshot and restored, so tuning leaves them unchanged.  best_ms (may be
  * NULL) receives the time per step. */
 int lbm_batch_tune(lbm_batch_t b, int trial_steps, float* best_ms);
@@ -333,7 +335,7 @@ int lbm_batch_step(lbm_batch_t b, long n);
 /* Steps per CUDA graph (even, 0..4096; 0 disables graphs). */
 int lbm_batch_set_graph_steps(lbm_batch_t b, int steps);
 
-/* Wait for the batch's queued work.  LBM_ECUDA also if a two-step launch
+/* Wait for the batch's queued work.  LBM_ECUDA also if a launch of several steps
  * timed out waiting for its tile load (the states are then invalid). */
 int lbm_batch_sync(lbm_batch_t b);
 
@@ -342,7 +344,8 @@ int lbm_batch_sync(lbm_batch_t b);
  * bodies of lbm_set_variant's variant 3, with its storage kind, edges, force and
  * rounding), so the populations cross HBM once per launch: four steps on 56 x 40
  * tiles if every lattice of the batch admits that (the cascaded collision, no
- * force, round to nearest), else two on 64 x 16 tiles.  Every lattice
+ * force, round to nearest) and the lattices' sizes suit those tiles, else two on
+ * 64 x 16 tiles.  Every lattice
  * gets a second population array (allocated here, kept by the lattice) and
  * the arrays trade roles at every launch.  lbm_batch_step then takes such
  * launches from even steps and single batched steps for an odd start or end; a

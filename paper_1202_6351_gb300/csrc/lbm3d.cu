@@ -26,9 +26,10 @@ constexpr int kStep3Threads = 128;
 // row: a row of 192 nodes in 128-wide blocks leaves a quarter of the lanes idle,
 // rows that do not fill a block in y idle warps.
 // FP32 storage is bound by HBM and load latency (216 B per update, 83 % of copy
-// bandwidth on 192^3), 16-bit storage by instruction issue: 758 instructions per
-// node on the even step and 920 on the odd one, 620 of them the collision; with
-// 64-bit slot offsets per population they were 873 and 1148.  The 27 slots of a
+// bandwidth on 192^3), 16-bit storage by instruction issue: on FP16 128^3 863 thread
+// instructions per node on the even step and 1026 on the odd one, most of them the
+// collision; with 64-bit slot offsets per population they were 926 and 1199 (FP32 192^3
+// now 808 and 971).  The 27 slots of a
 // node are nine row and three column offsets, kept in registers from load to
 // store: five blocks per SM (96 registers; FP32 192^3 us per step with four, five,
 // six, seven: 283, 271, 282, 321).

@@ -1,5 +1,5 @@
-// lbm_async.cuh -- the asynchronous-copy primitives of the two-steps-per-launch
-// kernel, as inline PTX: mbarrier set-up and bounded waits, the tiled tensor
+// lbm_async.cuh -- the asynchronous-copy primitives of the kernels that take several
+// steps per launch, as inline PTX: mbarrier set-up and bounded waits, the tiled tensor
 // load (TMA), the plain bulk copy shared -> global (bulk groups), and the
 // proxy fence between ordinary shared-memory writes and that copy.
 //

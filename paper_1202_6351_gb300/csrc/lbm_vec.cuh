@@ -259,11 +259,11 @@ __device__ __forceinline__ uint32_t enc_sr2(float2 v, unsigned r0, unsigned r1) 
 // byte permute), and the results replace the words they came from.
 //
 // Thread instructions per node 148 -> 104 (even step, 96 registers, 70 % of HBM
-// peak, bound by load latency) and 204 -> 184 (odd step: the narrow accesses of
+// peak, bound by load latency) and 204 -> 171 (odd step; with stochastic rounding 134 and 216: the narrow accesses of
 // the first and last lane of a warp, which every warp issues).  us per step,
 // before -> now: FP16 periodic 4096^2 114.6 -> 109.8, cavity 8192^2 464 -> 419,
-// cavity 1025^2 10.8 -> 9.5, BF16 4096^2 118.7 -> 108.0, FP16 stochastic 2048^2
-// 31.0 -> 30.5.  Gathering the narrow accesses of a side under one branch issued
+// cavity 1025^2 10.9 -> 9.5, BF16 4096^2 119.0 -> 107.7, FP16 stochastic 2048^2
+// 31.1 -> 31.0.  Gathering the narrow accesses of a side under one branch issued
 // as much and ran 2 % slower.
 template <int STORE, bool ODD, bool SR>
 __device__ __forceinline__ void step_vec_pair(const Args& a, int x0, int y, unsigned vmask, int lane) {

@@ -408,7 +408,7 @@ class Lattice:
 
 class Batch:
     """Many lattices advanced together (lbm_batch_*): one launch per step over
-    all their tiles, or one launch per two steps (set_two_step; the tuner may
+    all their tiles, or one per two or four steps (set_two_step; the tuner may
     choose either)."""
 
     POLICIES = {0: "round_robin", 1: "chunked", 2: "dynamic", 3: "one_cta_per_tile", 4: "two_steps_per_launch"}
@@ -453,7 +453,7 @@ class Batch:
         _check(self.lib.lbm_batch_set_graph_steps(self.b, int(steps)))
 
     def set_two_step(self, on=True):
-        """Two steps per launch for the whole batch (lbm_batch_set_two_step)."""
+        """Two or four steps per launch for the whole batch (lbm_batch_set_two_step)."""
         _check_alloc(self.lib.lbm_batch_set_two_step, self.b, 1 if on else 0)
         return self
 
